@@ -80,6 +80,9 @@ gks_status cuda_fail(gks_ctx *ctx, cudaError_t e, const char *where) {
     if (e_ != cudaSuccess) return cuda_fail(ctx, e_, #call); \
   } while (0)
 
+// Whether FP32 sums and reciprocals of eps are far from overflow and underflow.
+bool normal_eps(double v) { return v >= 0x1p-100 && v <= 0x1p100; }
+
 bool finite_positive(double v) { return std::isfinite(v) && v > 0.0; }
 
 // Fastest cleaning wave: gamma (psi, div B) and, in 3-D, chi (phi, div E); the 2-D TM system
@@ -431,12 +434,14 @@ gks_status gks_set_materials(gks_ctx *ctx, const double *eps, const double *mu) 
   if (mu && ctx->phm) return fail(ctx, GKS_E_UNSUPPORTED, "divergence cleaning needs mu = 1");
   // lattice speed: the fastest wave, light 1/sqrt(eps mu) or a cleaning wave (mu = 1)
   double cmax = cleaning_speed(ctx);
+  bool normal = true;
   for (int64_t i = 0; i < ctx->ncell; ++i) {
     const double e = eps[i], m = mu ? mu[i] : 1.0;
     if (!finite_positive(e) || !finite_positive(m))
       return fail(ctx, GKS_E_ARG, "eps and mu must be finite and > 0 (cell " +
                                       std::to_string(i) + ")");
     cmax = std::fmax(cmax, 1.0 / std::sqrt(e * m));
+    normal = normal && normal_eps(e);
   }
   gks_status s;
   if ((s = upload_cells(ctx, eps, 1, ctx->eps)) != GKS_OK) return s;
@@ -449,6 +454,7 @@ gks_status gks_set_materials(gks_ctx *ctx, const double *eps, const double *mu) 
     GKS_CUDA(cudaFreeAsync(ctx->mu, ctx->st));
     ctx->mu = nullptr;
   }
+  ctx->eps_normal = normal;
   ctx->c = ctx->c_user > 0 ? ctx->c_user : cmax;
   refresh_time_step(ctx);
   return GKS_OK;
@@ -464,13 +470,17 @@ gks_status gks_set_materials_box(gks_ctx *ctx, int64_t x0, int64_t x1, int64_t y
   if (!(ctx->c_user > 0))
     return fail(ctx, GKS_E_STATE, "a box update of eps needs a fixed lattice speed (c_lattice > 0)");
   const int64_t n = (x1 - x0) * (y1 - y0);
-  for (int64_t i = 0; i < n; ++i)
+  bool normal = ctx->eps_normal;
+  for (int64_t i = 0; i < n; ++i) {
     if (!finite_positive(eps_box[i]))
       return fail(ctx, GKS_E_ARG, "eps must be finite and > 0 (box entry " + std::to_string(i) + ")");
+    normal = normal && normal_eps(eps_box[i]);
+  }
   GKS_CUDA(cudaMemcpyAsync(ctx->staging, eps_box, sizeof(double) * (size_t)n,
                            cudaMemcpyHostToDevice, ctx->st));
   GKS_CUDA(gks::launch_box_to_cart(ctx->staging, ctx->eps, (int)x0, (int)(x1 - x0), (int)y0,
                                    (int)(y1 - y0), ctx->g.pitch, ctx->fp64, ctx->st));
+  ctx->eps_normal = normal;
   return GKS_OK;
 }
 
@@ -589,6 +599,7 @@ gks_status step_impl(gks_ctx *ctx, int64_t n_steps, const int win[4], bool objec
   a.c = ctx->c;
   a.flag = ctx->flag;
   a.limiter = ctx->limiter;
+  a.eps_normal = ctx->eps_normal;
   for (int64_t n = 0; n < n_steps; ++n) {
     const double t = ctx->t0 + (double)ctx->step * ctx->dt;
     a.src_amp = 0.0;

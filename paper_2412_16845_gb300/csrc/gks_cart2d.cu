@@ -1331,6 +1331,7 @@ cudaError_t launch_t(const CartGeom &g, const CartStepArgs &a, cudaStream_t st) 
 
 cudaError_t launch_cart2d_step(const CartGeom &g, const CartStepArgs &a, bool fp64,
                                cudaStream_t st) {
+  if (cart2d_tau0_supported(g, a, fp64)) return launch_cart2d_tau0(g, a, fp64, st);
   return fp64 ? launch_t<double>(g, a, st) : launch_t<float>(g, a, st);
 }
 

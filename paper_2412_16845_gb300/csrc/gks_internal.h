@@ -43,6 +43,7 @@ struct CartStepArgs {
   int *flag;            // non-finite flag (device)
   int window[4];        // x0, x1, y0, y1 (half open) of the cells to advance (2-D)
   int limiter = 0;      // GKS_LIMITER_*: slopes of the cell gradients
+  bool eps_normal = true;   // every eps lies in [2^-100, 2^100]
 };
 
 // Tetrahedral mesh geometry on the host (FP64; cells in internal Morton order).
@@ -131,6 +132,11 @@ cudaError_t launch_objective(const void *V, const int64_t *off, const double *w,
 // Launchers (return cudaGetLastError() of the launch).
 cudaError_t launch_cart2d_step(const CartGeom &g, const CartStepArgs &a, bool fp64,
                                cudaStream_t st);
+// 2-D step with tau = 0 and mu = 1 (gks_cart2d_tau0.cu); launch_cart2d_step dispatches to it when
+// cart2d_tau0_supported().
+bool cart2d_tau0_supported(const CartGeom &g, const CartStepArgs &a, bool fp64);
+cudaError_t launch_cart2d_tau0(const CartGeom &g, const CartStepArgs &a, bool fp64,
+                               cudaStream_t st);
 cudaError_t launch_cart3d_step(const CartGeom &g, const CartStepArgs &a, bool fp64,
                                cudaStream_t st);
 // FP32 3-D step with mu = 1, periodic or non-reflecting sides, no limiter (gks_cart3d_side.cu):
@@ -178,6 +184,7 @@ struct gks_ctx {
   void *V[2] = {nullptr, nullptr};
   int cur = 0;
   void *eps = nullptr;
+  bool eps_normal = true;       // every eps lies in [2^-100, 2^100]
   void *mu = nullptr;           // null: mu = 1
   void *src = nullptr;          // J_z mask or null
   int src_box[6] = {0, 0, 0, 0, 0, 0};

@@ -1,0 +1,79 @@
+"""GPU parity of the kernels for tau = 0 (the default kappa) with mu = 1 against the FP64 oracle, at the
+sizes where their tiles, strips and chunks begin and end.  Tolerances (relative L2) are those of every
+other path: FP64 <= 1e-12, FP32 <= 2e-5."""
+import numpy as np
+import pytest
+
+from paper_2412_16845_gb300 import workloads as wl
+from paper_2412_16845_gb300.gks import GKSSolver
+from tests.oracle_runs import oracle_cart_run, rel_l2
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"fp64": 1e-12, "fp32": 2e-5}
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    from paper_2412_16845_gb300 import build
+    build.build()
+
+
+def _grid(n, bc, seed, source=True, limiter=None, stretch=1.2):
+    rng = np.random.default_rng(seed)
+    cells = int(np.prod(n))
+    nc = 3 if len(n) == 2 else 6
+    mask = None
+    if source:
+        mask = np.zeros(cells)
+        at = rng.choice(cells, size=max(1, cells // 30), replace=False)
+        mask[at] = rng.uniform(-3, 3, at.size)
+    hi = tuple(v / n[0] * (stretch if a == 1 else 1.0) for a, v in enumerate(n))
+    return wl.CartWorkload(name="tau0", dim=len(n), n=n, lo=(0.0,) * len(n), hi=hi, bc=bc, cfl=0.4,
+                           steps=0, eps=rng.uniform(1.0, 4.0, cells), mu=None,
+                           fields0=rng.standard_normal((nc, cells)), jz_mask=mask,
+                           src=(1.0, 20.0, 0.02, 0.02), c_lattice=0.0, limiter=limiter)
+
+
+def _check(w, precision, steps):
+    s = GKSSolver.from_workload(w, precision=precision)
+    s.step(steps)
+    out = s.read_fields()
+    c = s.info()["c"]
+    s.close()
+    ref, _ = oracle_cart_run(w, steps, c=c)
+    assert rel_l2(out, ref) <= TOL[precision], rel_l2(out, ref)
+
+
+# 2-D: FP32 strips of 62 columns, four to a tile; FP64 strips of 30 or 62; chunks of 2 rows or more
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("n,bc", [
+    ((61, 5), "nnnn"), ((62, 2), "nnpp"), ((63, 1), "nnnn"), ((30, 33), "ppnn"), ((31, 3), "mmmm"),
+    ((248, 9), "nnnn"), ((249, 9), "nmnm"), ((247, 12), "mnpp"), ((310, 7), "ppmm"), ((125, 4), "pppp"),
+    ((2, 40), "mmnn"), ((1, 3), "nnnn"), ((3, 2), "pppp"), ((500, 70), "nnnn"),
+])
+def test_2d_tiles(n, bc, precision):
+    sides = tuple({"n": "nrbc", "p": "periodic", "m": "pec"}[b] for b in bc)
+    _check(_grid(n, sides, seed=n[0] + 7 * n[1]), precision, 9)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("n,bc", [((63, 9), "nrbc"), ((250, 6), "periodic"), ((130, 17), "pec")])
+def test_2d_limited_tiles(n, bc, precision):
+    _check(_grid(n, (bc,) * 4, seed=n[0], limiter="vanleer"), precision, 9)
+
+
+def test_2d_extreme_permittivity_keeps_its_results():
+    """eps beyond 2^+-100 leaves the FP32 tau = 0 kernel (its reciprocal needs normal numbers); FP64 is
+    the reference here, since the oracle's sums over velocities cancel at such eps."""
+    w = _grid((64, 20), ("nrbc",) * 4, seed=3, source=False)
+    w.eps[100] = 1e32
+    w.c_lattice = 1.0
+    out = {}
+    for precision in ("fp64", "fp32"):
+        s = GKSSolver.from_workload(w, precision=precision)
+        s.step(5)
+        out[precision] = s.read_fields()
+        s.close()
+    assert rel_l2(out["fp32"], out["fp64"]) <= 2e-5
+
