@@ -143,6 +143,9 @@ cudaError_t launch_cart3d_step(const CartGeom &g, const CartStepArgs &a, bool fp
 // the side-split flux; launch_cart3d_step dispatches to it when cart3d_side_supported().
 bool cart3d_side_supported(const CartGeom &g, const CartStepArgs &a, bool fp64);
 cudaError_t launch_cart3d_side(const CartGeom &g, const CartStepArgs &a, cudaStream_t st);
+// FP64 3-D step with tau = 0 and mu = 1 (gks_cart3d_tau0_f64.cu).
+bool cart3d_tau0_f64_supported(const CartStepArgs &a);
+cudaError_t launch_cart3d_tau0_f64(const CartGeom &g, const CartStepArgs &a, cudaStream_t st);
 // 2-D TM step with divergence cleaning (state Ez, Hx, Hy, psi; mu = 1).
 // Divergence-cleaning system on a 3-D grid: V = (E, H, phi, psi), 8 components.
 cudaError_t launch_cart3d_phm_step(const CartGeom &g, const CartStepArgs &a, double chi,

@@ -77,3 +77,14 @@ def test_2d_extreme_permittivity_keeps_its_results():
         s.close()
     assert rel_l2(out["fp32"], out["fp64"]) <= 2e-5
 
+
+# 3-D FP64: strips of 30 cells along any axis, up to 8 rows and any number of planes per warp
+@pytest.mark.parametrize("limiter", [None, "vanleer"])
+@pytest.mark.parametrize("n,bc", [
+    ((30, 9, 5), "nnnnnn"), ((31, 8, 3), "ppnnmm"), ((61, 3, 2), "mmppnn"), ((7, 30, 12), "nmnnpp"),
+    ((5, 6, 62), "pppppp"), ((1, 1, 1), "nnnnnn"), ((3, 17, 2), "nnppnm"), ((2, 2, 33), "mmmmmm"),
+])
+def test_3d_fp64_tiles(n, bc, limiter):
+    sides = tuple({"n": "nrbc", "p": "periodic", "m": "pec"}[b] for b in bc)
+    _check(_grid(n, sides, seed=sum(n), limiter=limiter), "fp64", 5)
+
