@@ -143,6 +143,9 @@ cudaError_t launch_cart3d_step(const CartGeom &g, const CartStepArgs &a, bool fp
 // the side-split flux; launch_cart3d_step dispatches to it when cart3d_side_supported().
 bool cart3d_side_supported(const CartGeom &g, const CartStepArgs &a, bool fp64);
 cudaError_t launch_cart3d_side(const CartGeom &g, const CartStepArgs &a, cudaStream_t st);
+// FP32 3-D step with tau = 0 where the side-split kernel would run (gks_cart3d_tau0.cu).
+bool cart3d_tau0_supported(const CartGeom &g, const CartStepArgs &a);
+cudaError_t launch_cart3d_tau0(const CartGeom &g, const CartStepArgs &a, cudaStream_t st);
 // FP64 3-D step with tau = 0 and mu = 1 (gks_cart3d_tau0_f64.cu).
 bool cart3d_tau0_f64_supported(const CartStepArgs &a);
 cudaError_t launch_cart3d_tau0_f64(const CartGeom &g, const CartStepArgs &a, cudaStream_t st);

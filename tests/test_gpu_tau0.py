@@ -88,3 +88,12 @@ def test_3d_fp64_tiles(n, bc, limiter):
     sides = tuple({"n": "nrbc", "p": "periodic", "m": "pec"}[b] for b in bc)
     _check(_grid(n, sides, seed=sum(n), limiter=limiter), "fp64", 5)
 
+
+# 3-D FP32: tiles of 64 columns x 10 rows, chunks of planes
+@pytest.mark.parametrize("n,bc", [
+    ((64, 10, 9), "nnnnnn"), ((65, 11, 3), "ppnnpp"), ((63, 21, 2), "nnppnn"), ((3, 2, 30), "nnnnnn"),
+    ((130, 9, 5), "pppppp"), ((1, 1, 1), "nnnnnn"), ((7, 12, 1), "nnnnpp"),
+])
+def test_3d_fp32_tiles(n, bc):
+    sides = tuple({"n": "nrbc", "p": "periodic"}[b] for b in bc)
+    _check(_grid(n, sides, seed=sum(n) + 1), "fp32", 7)
