@@ -148,7 +148,7 @@ gks_status setup_tets(gks_ctx *ctx, const gks_mesh_desc *d) {
     for (int a = 0; a < 3; ++a) { q[4 + a] = h.fdL[3 * f + a]; q[7 + a] = h.fdR[3 * f + a]; }
   }
   for (int64_t i = 0; i < h.nt; ++i) {
-    for (int k = 0; k < 12; ++k) cw[(size_t)i * gks::kTetCellW + k] = h.cw[12 * i + k];
+    for (int k = 0; k < 12; ++k) cw[(size_t)i * gks::kTetCellW + k] = 0.5 * h.cw[12 * i + k];
     for (int k = 0; k < 4; ++k)   // the face area enters here, not in the face pass
       cu[(size_t)i * gks::kTetCellU + k] =
           h.csign[4 * i + k] * h.farea[h.cface[4 * i + k]] * h.ivol[i];

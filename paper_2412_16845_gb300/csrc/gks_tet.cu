@@ -17,7 +17,11 @@
 namespace gks {
 namespace {
 
-constexpr int TB = 256;
+// Threads per block: FP64 passes are bound by the FP64 pipe, one warp fills a scheduler's, and small
+// blocks even out the last wave (48,000 tets: 256 threads 762, 128 threads 721, 64 threads 719 us for
+// ten steps); FP32 passes are bound by gathers.
+template <typename T>
+constexpr int TBT = sizeof(T) == 4 ? 256 : 64;
 
 // Reciprocals: FP32 uses the fast hardware reciprocal (about 1 ulp), FP64 divides.
 __device__ __forceinline__ float trcp(float x) { return __fdividef(1.f, x); }
@@ -25,12 +29,13 @@ __device__ __forceinline__ double trcp(double x) { return 1.0 / x; }
 __device__ __forceinline__ float trcp2(float x) { return __fdividef(2.f, x); }
 __device__ __forceinline__ double trcp2(double x) { return 2.0 / x; }
 
+template <typename T>
 int blocks_for(int64_t n) {
-  int64_t b = (n + TB - 1) / TB;
+  const int64_t b = (n + TBT<T> - 1) / TBT<T>;
   return (int)(b < 1 ? 1 : b);
 }
 
-// The twelve gradient weights n|l|/|Omega| of a cell (its four faces): vector loads.
+// The twelve gradient weights n|l|/(2|Omega|) of a cell (its four faces): vector loads.
 __device__ __forceinline__ void load_cell_w(const float *p, float w[kTetCellW]) {
 #pragma unroll
   for (int k = 0; k < kTetCellW / 4; ++k) {
@@ -50,7 +55,7 @@ template <typename T>
 __global__ void tet_gradient_kernel(const T *__restrict__ V, const int32_t *__restrict__ cnb,
                                     const T *__restrict__ cw, int64_t nt, int pec,
                                     T *__restrict__ G) {
-  const int64_t i = blockIdx.x * (int64_t)TB + threadIdx.x;
+  const int64_t i = blockIdx.x * (int64_t)TBT<T> + threadIdx.x;
   if (i >= nt) return;
   // every load is issued before the arithmetic: the four neighbour indices in one vector load,
   // then the 24 neighbour values (a wall face reads the cell itself), so that the gathers are in
@@ -67,39 +72,29 @@ __global__ void tet_gradient_kernel(const T *__restrict__ V, const int32_t *__re
     for (int c = 0; c < 6; ++c) vn[k][c] = V[c * nt + j];
   }
   load_cell_w(cw + kTetCellW * i, w);
+  // sum over the faces of (V_i + V_k)/2 n|l|/|Omega|: the weights of a cell add up to zero, so V_i
+  // drops out and the sum is that of V_k w_k (w_k holds the 1/2): 72 operations instead of 120
   T g[3][6];
 #pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int c = 0; c < 6; ++c) g[a][c] = T(0);
-#pragma unroll
   for (int k = 0; k < 4; ++k) {
-    T vf[6];
-    if (nb[k] >= 0) {
-#pragma unroll
-      for (int c = 0; c < 6; ++c) vf[c] = T(0.5) * (vi[c] + vn[k][c]);
-    } else if (pec) {
-      // PEC wall: face value (V + P V)/2 of the mirror ghost P V = (-E + 2 (E.n) n, H - 2 (H.n) n),
-      // i.e. the normal part of E and the tangential part of H
+    if (nb[k] < 0 && pec) {
+      // PEC wall: V_k is the mirror ghost P V = (-E + 2 (E.n) n, H - 2 (H.n) n)
       const T *wk = w + 3 * k;
       const T inv = T(1) / sqrt(wk[0] * wk[0] + wk[1] * wk[1] + wk[2] * wk[2]);
       const T n[3] = {wk[0] * inv, wk[1] * inv, wk[2] * inv};
-      const T en = vi[0] * n[0] + vi[1] * n[1] + vi[2] * n[2];
-      const T hn = vi[3] * n[0] + vi[4] * n[1] + vi[5] * n[2];
+      const T en = T(2) * (vi[0] * n[0] + vi[1] * n[1] + vi[2] * n[2]);
+      const T hn = T(2) * (vi[3] * n[0] + vi[4] * n[1] + vi[5] * n[2]);
 #pragma unroll
       for (int a = 0; a < 3; ++a) {
-        vf[a] = en * n[a];
-        vf[3 + a] = vi[3 + a] - hn * n[a];
+        vn[k][a] = en * n[a] - vi[a];
+        vn[k][3 + a] = vi[3 + a] - hn * n[a];
       }
-    } else {
-#pragma unroll
-      for (int c = 0; c < 6; ++c) vf[c] = vi[c];
     }
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       const T wa = w[3 * k + a];
 #pragma unroll
-      for (int c = 0; c < 6; ++c) g[a][c] += vf[c] * wa;
+      for (int c = 0; c < 6; ++c) g[a][c] = k == 0 ? vn[k][c] * wa : g[a][c] + vn[k][c] * wa;
     }
   }
 #pragma unroll
@@ -181,13 +176,13 @@ __device__ __forceinline__ Side3<T> pec_ghost(const Side3<T> &l) {
 // FP32 with mu = 1: capped at 64 registers (no spills) for 4 CTAs per SM; the gathers' latency is
 // hidden by more resident warps (3.7% faster than at 72 registers).
 template <typename T, bool HAS_MU>
-__global__ void __launch_bounds__(TB, (sizeof(T) == 4 && !HAS_MU) ? 4 : 1)
+__global__ void __launch_bounds__(TBT<T>, (sizeof(T) == 4 && !HAS_MU) ? 4 : 1)
     tet_face_kernel(const T *__restrict__ V, const T *__restrict__ G,
                                 const T *__restrict__ eps, const T *__restrict__ mu,
                                 const int32_t *__restrict__ fL, const int32_t *__restrict__ fR,
                                 const T *__restrict__ fgeo, int64_t nt, int64_t nf, int pec,
                                 const K3<T> K, const F3K<T> FK, T *__restrict__ F) {
-  const int64_t f = blockIdx.x * (int64_t)TB + threadIdx.x;
+  const int64_t f = blockIdx.x * (int64_t)TBT<T> + threadIdx.x;
   if (f >= nf) return;
   T q[kTetFaceGeo];
   load_face_geo(fgeo + kTetFaceGeo * f, q);
@@ -227,6 +222,95 @@ __global__ void __launch_bounds__(TB, (sizeof(T) == 4 && !HAS_MU) ? 4 : 1)
           Tm[a] * loc[3 * b] + Tm[3 + a] * loc[3 * b + 1] + Tm[6 + a] * loc[3 * b + 2];
 }
 
+// Constants of the tau = 0 face flux: C1/2, C3/2 and 1/c.
+template <typename T>
+struct TetK0 {
+  T h1, h3, ic;
+};
+
+// A side's share of the tau = 0 face flux (see tet_face_tau0_kernel), added into PE, QE, QH; m = n/c
+// for the low side, -n/c for the high side.  The gradient rows are loaded a field at a time.
+template <typename T>
+__device__ __forceinline__ void tet_side_tau0(const T *__restrict__ V, const T *__restrict__ G, T eps,
+                                              int64_t nt, int64_t cell, const T d[3], const T m[3],
+                                              const TetK0<T> &K, T PE[3], T QE[3], T QH[3]) {
+  const T m1[3] = {K.h1 * m[0], K.h1 * m[1], K.h1 * m[2]};
+  const T m3[3] = {K.h3 * m[0], K.h3 * m[1], K.h3 * m[2]};
+  const T e1 = K.h1 * eps;
+  T v[6], g[3][6];
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int c = 0; c < 6; ++c) g[a][c] = G[(6 * a + c) * nt + cell];
+#pragma unroll
+  for (int c = 0; c < 6; ++c)
+    v[c] = V[c * nt + cell] + d[0] * g[0][c] + d[1] * g[1][c] + d[2] * g[2][c];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int b = (a + 1) % 3, c = (a + 2) % 3;
+    PE[a] += v[3 + a] + (m[b] * v[c] - m[c] * v[b]);                       // H + m x E
+    QE[a] += eps * (g[b][c] - g[c][b]);                                    // eps curl E
+    QE[a] += m[0] * g[0][3 + a] + m[1] * g[1][3 + a] + m[2] * g[2][3 + a]; // (m . grad) H
+    QH[a] += e1 * v[a] - (m1[b] * v[3 + c] - m1[c] * v[3 + b]);            // eps E - m x H
+    QH[a] += K.h3 * (g[b][3 + c] - g[c][3 + b]);                           // curl H
+    QH[a] -= m3[0] * g[0][a] + m3[1] * g[1][a] + m3[2] * g[2][a];          // (m . grad) E
+  }
+}
+
+// Face pass for tau = 0 (Sec. 4.1) and mu = 1, without face frames.  Only C1 <u g0> + C3 <u g_t> is
+// left of the flux; with F_n(E, H) = (-n x H, n x E), V0_t = (ie curl H0, -curl E0) and
+// n x curl(n x a) = -n x (n . grad) a it is a tangential vector in global components,
+//   F_E = n x (-C1/2 PE + C3/2 ie QE),   F_H = ie n x QH,   ie = 1/eps_s,   s = +-1 (low, high side)
+//   PE = sum H + s n x E / c,    QE = sum eps curl E + s (n . grad) H / c
+//   QH = sum C1/2 (eps E - s n x H / c) + C3/2 (curl H - s (n . grad) E / c)
+// : 165 operations a face where rotating both sides' 24 values into the face frame took 520.  A
+// non-reflecting ghost adds nothing and ie = 1/eps; at a PEC wall the mirror image doubles PE and QE
+// (tangentially) and cancels QH.
+template <typename T>
+__global__ void __launch_bounds__(TBT<T>, sizeof(T) == 4 ? 4 : 1)
+    tet_face_tau0_kernel(const T *__restrict__ V, const T *__restrict__ G,
+                         const T *__restrict__ eps, const int32_t *__restrict__ fL,
+                         const int32_t *__restrict__ fR, const T *__restrict__ fgeo, int64_t nt,
+                         int64_t nf, int pec, const TetK0<T> K, T *__restrict__ F) {
+  const int64_t f = blockIdx.x * (int64_t)TBT<T> + threadIdx.x;
+  if (f >= nf) return;
+  const int32_t L = fL[f], R = fR[f];
+  T q[kTetFaceGeo];
+  load_face_geo(fgeo + kTetFaceGeo * f, q);
+  const T *n = q;
+  T m[3] = {K.ic * n[0], K.ic * n[1], K.ic * n[2]};
+  T PE[3] = {T(0), T(0), T(0)}, QE[3] = {T(0), T(0), T(0)}, QH[3] = {T(0), T(0), T(0)};
+  const T el = eps[L];
+  tet_side_tau0<T>(V, G, el, nt, L, q + 4, m, K, PE, QE, QH);
+  T ie;
+  if (R >= 0) {
+    const T er = eps[R];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) m[a] = -m[a];
+    tet_side_tau0<T>(V, G, er, nt, R, q + 7, m, K, PE, QE, QH);
+    ie = trcp2(el + er);
+  } else {
+    ie = trcp(el);
+    if (pec) {
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        PE[a] *= T(2);
+        QE[a] *= T(2);
+        QH[a] = T(0);
+      }
+    }
+  }
+  const T k3 = K.h3 * ie;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) PE[a] = k3 * QE[a] - K.h1 * PE[a];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const int b = (a + 1) % 3, c = (a + 2) % 3;
+    F[a * nf + f] = n[b] * PE[c] - n[c] * PE[b];
+    F[(3 + a) * nf + f] = ie * (n[b] * QH[c] - n[c] * QH[b]);
+  }
+}
+
 // The four update weights sign_k / |Omega| of a cell: one vector load (FP32) or two (FP64).
 __device__ __forceinline__ void load_cell_u(const float *p, float w[4]) {
   const float4 v = __ldg(reinterpret_cast<const float4 *>(p));
@@ -246,7 +330,7 @@ __global__ void tet_update_kernel(const T *__restrict__ V, T *__restrict__ Vout,
                                   const T *__restrict__ cu, const T *__restrict__ F, int64_t nt,
                                   int64_t nf,
                                   int *__restrict__ flag) {
-  const int64_t i = blockIdx.x * (int64_t)TB + threadIdx.x;
+  const int64_t i = blockIdx.x * (int64_t)TBT<T> + threadIdx.x;
   bool bad = false;
   if (i < nt) {
     T w[4];
@@ -344,17 +428,26 @@ cudaError_t step_t(const TetDev &g, const void *Vin, void *Vout, const void *eps
   T *F = static_cast<T *>(g.Fscratch);
   const T *fgeo = static_cast<const T *>(g.fgeo);
   const T *cw = static_cast<const T *>(g.cw), *cu = static_cast<const T *>(g.cu);
-  tet_gradient_kernel<T><<<blocks_for(g.nt), TB, 0, st>>>(V, g.cnb, cw, g.nt, g.pec, G);
+  tet_gradient_kernel<T><<<blocks_for<T>(g.nt), TBT<T>, 0, st>>>(V, g.cnb, cw, g.nt, g.pec, G);
+  if (!mu && C[1] == 0.0 && C[3] == 0.0 && C[4] == 0.0) {
+    const TetK0<T> K0 = {T(0.5 * C[0]), T(0.5 * C[2]), T(1.0 / c)};
+    tet_face_tau0_kernel<T><<<blocks_for<T>(g.nf), TBT<T>, 0, st>>>(
+        V, G, static_cast<const T *>(eps), g.fL, g.fR, fgeo, g.nt, g.nf, g.pec, K0, F);
+    tet_update_kernel<T><<<blocks_for<T>(g.nt), TBT<T>, 0, st>>>(
+        V, static_cast<T *>(Vout), static_cast<const T *>(eps), nullptr,
+        static_cast<const T *>(src), T(src_amp), g.cface, cu, F, g.nt, g.nf, flag);
+    return cudaGetLastError();
+  }
   const K3<T> K = make_k3<T>(C, 1.0, c);     // fluxes carry dt (C_i), areas applied per face
   const F3K<T> FK = make_f3k<T>(C, 1.0, c);
   if (mu)
-    tet_face_kernel<T, true><<<blocks_for(g.nf), TB, 0, st>>>(
+    tet_face_kernel<T, true><<<blocks_for<T>(g.nf), TBT<T>, 0, st>>>(
         V, G, static_cast<const T *>(eps), static_cast<const T *>(mu), g.fL, g.fR, fgeo, g.nt,
         g.nf, g.pec, K, FK, F);
   else
-    tet_face_kernel<T, false><<<blocks_for(g.nf), TB, 0, st>>>(
+    tet_face_kernel<T, false><<<blocks_for<T>(g.nf), TBT<T>, 0, st>>>(
         V, G, static_cast<const T *>(eps), nullptr, g.fL, g.fR, fgeo, g.nt, g.nf, g.pec, K, FK, F);
-  tet_update_kernel<T><<<blocks_for(g.nt), TB, 0, st>>>(
+  tet_update_kernel<T><<<blocks_for<T>(g.nt), TBT<T>, 0, st>>>(
       V, static_cast<T *>(Vout), static_cast<const T *>(eps), static_cast<const T *>(mu),
       static_cast<const T *>(src), T(src_amp), g.cface, cu, F, g.nt, g.nf, flag);
   return cudaGetLastError();
