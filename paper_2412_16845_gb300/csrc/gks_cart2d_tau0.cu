@@ -19,7 +19,7 @@
 //  * FP32 (cart2d_tau0_kernel): instruction issue and HBM.  About 54 paired FP32 instructions per
 //    two cells; the general flux takes 132.
 //  * FP64 (cart2d_tau0_f64_kernel): the FP64 pipe.  A GB300 issues one FP64 warp instruction per
-//    64 cycles and scheduler (measured), so the count of FP64 operations, 51 and three divisions a
+//    64 cycles and scheduler (measured), so the count of FP64 operations, 51 and three reciprocals a
 //    cell, and an even spread of rows over the 608 schedulers are the whole time.
 #include <cuda_runtime.h>
 
@@ -28,6 +28,7 @@
 
 #include "gks_flux2.cuh"
 #include "gks_internal.h"
+#include "gks_rcp.cuh"
 #include "gks_tma.cuh"
 
 namespace gks {
@@ -44,13 +45,6 @@ __device__ __forceinline__ f2 vmul(f2 a, f2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ f2 vmul(float k, f2 b) { return __fmul2_rn(pk(k, k), b); }
 __device__ __forceinline__ f2 vfma(f2 a, f2 b, f2 c) { return __ffma2_rn(a, b, c); }
 __device__ __forceinline__ f2 vfma(float k, f2 b, f2 c) { return __ffma2_rn(pk(k, k), b, c); }
-// 1 / s by the hardware reciprocal (1 ulp): the launch rule keeps s within 2^+-100, where it needs
-// none of the scaling that __fdividef adds for subnormal and huge divisors (6 instructions a value)
-__device__ __forceinline__ float rcp_normal(float s) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(s));
-  return r;
-}
 __device__ __forceinline__ f2 vrcp(f2 s) { return pk(rcp_normal(s.x), rcp_normal(s.y)); }
 
 // The columns of one lane in FP64: 32 apart.
@@ -68,7 +62,7 @@ template <int NC> __device__ __forceinline__ DV<NC> vmul(const DV<NC> &a, const 
 template <int NC> __device__ __forceinline__ DV<NC> vmul(double k, const DV<NC> &b) { GKS_DV(k * b.v[i]); }
 template <int NC> __device__ __forceinline__ DV<NC> vfma(const DV<NC> &a, const DV<NC> &b, const DV<NC> &c) { GKS_DV(fma(a.v[i], b.v[i], c.v[i])); }
 template <int NC> __device__ __forceinline__ DV<NC> vfma(double k, const DV<NC> &b, const DV<NC> &c) { GKS_DV(fma(k, b.v[i], c.v[i])); }
-template <int NC> __device__ __forceinline__ DV<NC> vrcp(const DV<NC> &a) { GKS_DV(1.0 / a.v[i]); }
+template <int NC> __device__ __forceinline__ DV<NC> vrcp(const DV<NC> &a) { GKS_DV(rcp_normal(a.v[i])); }
 #undef GKS_DV
 
 template <bool LIMIT>
@@ -745,10 +739,11 @@ cudaError_t launch_f64(const CartGeom &g, const CartStepArgs &a, cudaStream_t st
 }  // namespace
 
 bool cart2d_tau0_supported(const CartGeom &g, const CartStepArgs &a, bool fp64) {
-  if (a.mu || a.C[1] != 0.0 || a.C[3] != 0.0 || a.C[4] != 0.0 || !(a.C[0] > 0.0)) return false;
+  // (the reciprocals of eps are those of gks_rcp.cuh)
+  if (a.mu || a.C[1] != 0.0 || a.C[3] != 0.0 || a.C[4] != 0.0 || !(a.C[0] > 0.0) || !a.eps_normal)
+    return false;
   if (fp64) return true;
-  // FP32 takes the hardware reciprocal of eps; its staged rows wrap by one period
-  if (!a.eps_normal || (g.periodic[1] && g.ny < 2)) return false;
+  if (g.periodic[1] && g.ny < 2) return false;        // FP32: the staged rows wrap by one period
   return tensor_map_encoder() != nullptr;
 }
 

@@ -4,7 +4,7 @@
 // The march is that of cart3d_side_kernel (gks_cart3d_side.cu, which keeps tau > 0): a CTA owns 64
 // columns x NWO rows of a chunk of z-planes; a row warp holds two adjacent cells per lane as the
 // halves of a float2; two halo warps supply the y-sides of the rows below and above and, a plane
-// ahead, the x-sides of the columns left and right of the tile; planes arrive by TMA into five slots.
+// ahead, the x-sides of the columns left and right of the tile; planes arrive by TMA into four slots.
 // With tau = 0 a cell sends 6 values to a neighbour instead of 12 and a face carries 4 components
 // instead of 6: 81 paired instructions a cell pair's worth of flux and update instead of 220, half the
 // shuffles and shared-memory exchange, and the z-sides fit in registers (no tensor memory).
@@ -13,22 +13,21 @@
 
 #include "gks_internal.h"
 #include "gks_pair3.cuh"
+#include "gks_rcp.cuh"
 #include "gks_tma.cuh"
 
 namespace gks {
 namespace {
 
-#ifndef GKS_T3_NWO
-#define GKS_T3_NWO 10
-#endif
-constexpr int NWO = GKS_T3_NWO;         // row warps per CTA
+constexpr int NWO = 10;                 // row warps per CTA
 constexpr int NWARP = NWO + 2;          // plus the halo warps H0 (below) and H1 (above)
 constexpr int NTH = NWARP * 32;
+constexpr int CTAS = 1;                 // per SM
 constexpr int TCOLS = 64;               // columns per CTA (two per lane)
 constexpr int TW = 72;                  // staged columns X0-4 .. X0+67 (16-byte chunks)
 constexpr int NR = NWO + 4;             // staged rows y0-2 .. y0+NWO+1
 constexpr int NA = 7;                   // staged arrays: Ex, Ey, Ez, Hx, Hy, Hz, eps
-constexpr int NSLOT = 5;
+constexpr int NSLOT = 4;
 constexpr unsigned FULL = 0xffffffffu;
 // wrapped entries of a staged plane on periodic sides: two layers beyond each side, every row
 // for columns and every column for rows, all arrays
@@ -37,12 +36,6 @@ constexpr int kMaxFix = NA * (4 * NR + 4 * TW);
 using f2 = float2;
 
 __device__ __forceinline__ f2 pk(float a, float b) { return make_float2(a, b); }
-// 1 / s by the hardware reciprocal (1 ulp); the launch rule keeps eps within 2^+-100
-__device__ __forceinline__ float rcp_normal(float s) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(s));
-  return r;
-}
 __device__ __forceinline__ f2 vrcp(f2 s) { return pk(rcp_normal(s.x), rcp_normal(s.y)); }
 
 // Paired FP32 arithmetic (two cells per value); a constant is a scalar kernel parameter replicated
@@ -271,7 +264,7 @@ __device__ __forceinline__ void zero6(Sides3<f2> &a) {
   for (int m = 0; m < 6; ++m) a.v[m] = pk(0.f, 0.f);
 }
 
-__global__ void __launch_bounds__(NTH, 1)
+__global__ void __launch_bounds__(NTH, CTAS)
     cart3d_tau0_kernel(const __grid_constant__ CUtensorMap tmV,
                        const __grid_constant__ CUtensorMap tmE, const __grid_constant__ Args a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -345,7 +338,6 @@ __global__ void __launch_bounds__(NTH, 1)
   }
   __syncthreads();
   if (s.err) return;                                          // nothing else is in flight
-  if (issuer) tma_plane(s, &tmV, &tmE, slot_of(z0 + 3), X0 - 4, y0 - 2, zidx(z0 + 3));
 
   f2 W0[7], Wp[7];                      // own pair at planes k, k+1 (Wm: k-1)
   f2 B[6], Minv = pk(0.f, 0.f);         // pending update of plane k-1 (z-face components)
@@ -390,8 +382,8 @@ __global__ void __launch_bounds__(NTH, 1)
 #pragma unroll 1
   for (int k = z0; k <= z1; ++k) {
     const bool last = k == z1;                 // only the z-face below plane z1 remains
-    if (issuer && !last && k + 4 <= z1 + 1)
-      tma_plane(s, &tmV, &tmE, slot_of(k + 4), X0 - 4, y0 - 2, zidx(k + 4));
+    if (issuer && k + 3 <= last_plane)         // plane k-1's slot is free
+      tma_plane(s, &tmV, &tmE, slot_of(k + 3), X0 - 4, y0 - 2, zidx(k + 3));
     const int s0 = slot_of(k), sp = slot_of(k + 1);
     load_pair(s, sp, q, Wp);
     f2 acc[6];
@@ -538,10 +530,7 @@ __global__ void __launch_bounds__(NTH, 1)
       }
     }
     __syncthreads();                            // B2: face fluxes; plane k+3 visible
-    if (s.err) {                                // leave together; wait (bounded) for the copy
-      if (k + 4 <= last_plane) mbar_wait(&s.bar[slot_of(k + 4)], parity_of(k + 4));
-      break;
-    }
+    if (s.err) break;                           // leave together; no copy is in flight
     if (owned) {
       const int below = warp == 0 ? NWO : warp - 1;
 #pragma unroll
@@ -616,7 +605,7 @@ cudaError_t launch_cart3d_tau0(const CartGeom &g, const CartStepArgs &a, cudaStr
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (sms <= 0) sms = 1;
+    sms = sms > 0 ? sms * CTAS : 1;
   }
   // z chunks: one CTA per SM; pick the chunk count that fills whole waves best.  A CTA's fixed
   // cost -- staging its first four planes with nothing to overlap them, the z-vectors of the

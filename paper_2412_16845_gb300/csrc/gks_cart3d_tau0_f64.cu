@@ -3,7 +3,7 @@
 //
 // Bound: the FP64 pipe.  A GB300 issues one FP64 warp instruction per 64 cycles and scheduler
 // (measured; one warp with independent instructions fills it), so the time is the number of FP64
-// operations (162 and four divisions a cell; the general kernel runs 763) times how unevenly they
+// operations (162 and four reciprocals a cell; the general kernel runs 763) times how unevenly they
 // are spread over the 608 schedulers.  Everything else -- loads, shuffles, shared memory, index
 // arithmetic, uncoalesced access -- has 64 issue slots per FP64 instruction and is free.
 //
@@ -22,6 +22,7 @@
 #include "gks_flux2.cuh"
 #include "gks_internal.h"
 #include "gks_pair3.cuh"
+#include "gks_rcp.cuh"
 
 namespace gks {
 namespace {
@@ -171,7 +172,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2) cart3d_tau0_f64_kernel(const __
         if (gx) l.v[i] = r.v[i] = 0.0;
         l.v[i] = __shfl_sync(FULL, l.v[i], lprev);
       }
-      const double inv = 1.0 / (__shfl_sync(FULL, eps, lprev) + eps);
+      const double inv = rcp_normal(__shfl_sync(FULL, eps, lprev) + eps);
       face3<OpD>(l, r, inv, p.k[0], G);
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
@@ -195,7 +196,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2) cart3d_tau0_f64_kernel(const __
         for (int i = 0; i < 6; ++i) l.v[i] = r.v[i] = 0.0;
       }
       if constexpr (WHAT != ROWLO) {                  // face between rows j-1 and j
-        face3<OpD>(yl, r, 1.0 / (epsr + eps), p.k[1], G);
+        face3<OpD>(yl, r, rcp_normal(epsr + eps), p.k[1], G);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const double s = (i & 1) ? p.k[1][i / 2].sH : p.k[1][i / 2].sE;
@@ -224,7 +225,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2) cart3d_tau0_f64_kernel(const __
         for (int i = 0; i < 6; ++i) zl.v[i] = q[i * 32];
         const int64_t om = ax.o + bj.o + cm.o;
         const double epsm = __ldg(p.eps + om);
-        face3<OpD>(zl, r, 1.0 / (epsm + eps), p.k[2], G);
+        face3<OpD>(zl, r, rcp_normal(epsm + eps), p.k[2], G);
         if (k > k0) {                                 // completes plane k-1
           double nv[6];
 #pragma unroll
@@ -233,7 +234,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2) cart3d_tau0_f64_kernel(const __
           for (int i = 0; i < 4; ++i)
             nv[face_comp<2>(i)] = fma(-((i & 1) ? p.k[2][i / 2].sH : p.k[2][i / 2].sE), G[i],
                                       nv[face_comp<2>(i)]);
-          const double ie = 1.0 / epsm;
+          const double ie = rcp_normal(epsm);
 #pragma unroll
           for (int c = 0; c < 3; ++c) nv[c] = fma(nv[c], ie, __ldg(p.F[c] + om));
           if (store) {
@@ -280,7 +281,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2) cart3d_tau0_f64_kernel(const __
 }  // namespace
 
 bool cart3d_tau0_f64_supported(const CartStepArgs &a) {
-  return !a.mu && a.C[1] == 0.0 && a.C[3] == 0.0 && a.C[4] == 0.0 && a.C[0] > 0.0;
+  return !a.mu && a.eps_normal && a.C[1] == 0.0 && a.C[3] == 0.0 && a.C[4] == 0.0 && a.C[0] > 0.0;
 }
 
 cudaError_t launch_cart3d_tau0_f64(const CartGeom &g, const CartStepArgs &a, cudaStream_t st) {
@@ -299,7 +300,7 @@ cudaError_t launch_cart3d_tau0_f64(const CartGeom &g, const CartStepArgs &a, cud
   const int n[3] = {g.nx, g.ny, g.nz};
   const int64_t stride[3] = {1, g.pitch, g.plane};
   // Lane axis, rows per warp and planes per chunk: the least FP64 work on the busiest scheduler for
-  // one to four warps on each.  A chunk costs about 0.35 of a row (plane) more; one warp alone on a
+  // one to four warps on each.  A chunk costs about 0.48 of a row (plane) more; one warp alone on a
   // scheduler does not hide its loads (an eighth); strided access along the lanes costs a few
   // percent.
   const int64_t sched = (int64_t)sms * WARPS;
@@ -314,8 +315,8 @@ cudaError_t launch_cart3d_tau0_f64(const CartGeom &g, const CartStepArgs &a, cud
         const int64_t want = std::max<int64_t>(1, m * sched / ((int64_t)strips * nrow));
         const int Z = (int)((nm + want - 1) / want), nmarch = (nm + Z - 1) / Z;
         const int64_t nw = (int64_t)strips * nrow * nmarch;
-        const double cost = (double)((nw + sched - 1) / sched) * (R + 0.35) * (Z + 0.35) *
-                            (nw > sched ? 1.0 : 1.125) * (ax == 0 ? 1.0 : 1.04);
+        const double cost = (double)((nw + sched - 1) / sched) * (R + 0.48) * (Z + 0.48) *
+                            (nw > sched ? 1.0 : 1.125) * (ax == 0 ? 1.0 : 1.25);
         if (cost < best * 0.999) {
           best = cost;
           lane_axis = ax;
