@@ -600,21 +600,35 @@ gks_status step_impl(gks_ctx *ctx, int64_t n_steps, const int win[4], bool objec
   a.flag = ctx->flag;
   a.limiter = ctx->limiter;
   a.eps_normal = ctx->eps_normal;
-  for (int64_t n = 0; n < n_steps; ++n) {
-    const double t = ctx->t0 + (double)ctx->step * ctx->dt;
-    a.src_amp = 0.0;
-    if (ctx->src) {
-      const double tt = t - ctx->srcT0;
-      if (ctx->srcKind == 1)
-        a.src_amp = tt >= 0.0 ? ctx->dt * ctx->srcA * std::cos(2.0 * M_PI * ctx->srcF0 * tt) : 0.0;
-      else
-        a.src_amp = ctx->dt * ctx->srcA * std::exp(-(tt / ctx->srcS) * (tt / ctx->srcS)) *
-                    std::sin(2.0 * M_PI * ctx->srcF0 * tt);
-    }
+  // dt times the source's waveform at step `step`
+  auto amplitude = [ctx](int64_t step) {
+    if (!ctx->src) return 0.0;
+    const double t = ctx->t0 + (double)step * ctx->dt, tt = t - ctx->srcT0;
+    if (ctx->srcKind == 1)
+      return tt >= 0.0 ? ctx->dt * ctx->srcA * std::cos(2.0 * M_PI * ctx->srcF0 * tt) : 0.0;
+    return ctx->dt * ctx->srcA * std::exp(-(tt / ctx->srcS) * (tt / ctx->srcS)) *
+           std::sin(2.0 * M_PI * ctx->srcF0 * tt);
+  };
+  // windowed steps (objective = false) march: their windows are recomputed step by step
+  const bool small = objective && ctx->kind == GKS_CARTESIAN && ctx->dim == 2 && !ctx->phm;
+  const bool probe = objective && ctx->np > 0;       // needs the state after every step
+  gks::SmallPlan pl;
+  if (small) pl = gks::cart2d_small_plan(ctx->g, a, ctx->fp64, probe ? 1 : n_steps);
+  for (int64_t n = 0; n < n_steps;) {
+    a.src_amp = amplitude(ctx->step);
     a.V = ctx->V[ctx->cur];
     a.Vout = ctx->V[ctx->cur ^ 1];
     cudaError_t e;
-    if (ctx->kind == GKS_TET) {
+    int done = 1;
+    if (pl.steps > n_steps - n)                       // the last launch takes fewer steps
+      pl = gks::cart2d_small_plan(ctx->g, a, ctx->fp64, n_steps - n);
+    if (pl.steps > 0) {
+      double amp[gks::kSmallSteps];
+      done = pl.steps;
+      for (int s = 0; s < done; ++s) amp[s] = amplitude(ctx->step + s);
+      e = gks::launch_cart2d_small(ctx->g, a, pl, amp, ctx->fp64, ctx->st);
+      ctx->launches += 1;
+    } else if (ctx->kind == GKS_TET) {
       e = gks::launch_tet_step(ctx->tet, a.V, a.Vout, a.eps, a.mu, a.src, a.src_amp, a.C, a.c,
                                a.flag, ctx->fp64, ctx->st);
       ctx->launches += 3;
@@ -630,8 +644,9 @@ gks_status step_impl(gks_ctx *ctx, int64_t n_steps, const int win[4], bool objec
     }
     if (e != cudaSuccess) return cuda_fail(ctx, e, "step launch");
     ctx->cur ^= 1;
-    ctx->step += 1;
-    if (objective && ctx->np > 0) {
+    ctx->step += done;
+    n += done;
+    if (probe) {
       e = gks::launch_objective(ctx->V[ctx->cur], ctx->probe_off, ctx->probe_w, ctx->np, ctx->dt,
                                 ctx->obj, ctx->fp64, ctx->st);
       if (e != cudaSuccess) return cuda_fail(ctx, e, "objective launch");

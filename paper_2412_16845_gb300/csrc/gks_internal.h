@@ -143,6 +143,17 @@ cudaError_t launch_cart3d_step(const CartGeom &g, const CartStepArgs &a, bool fp
 // the side-split flux; launch_cart3d_step dispatches to it when cart3d_side_supported().
 bool cart3d_side_supported(const CartGeom &g, const CartStepArgs &a, bool fp64);
 cudaError_t launch_cart3d_side(const CartGeom &g, const CartStepArgs &a, cudaStream_t st);
+// Several 2-D steps in one launch on grids too small to fill the GPU (gks_cart2d_small.cu): the tile
+// and steps per launch (0: the marching kernels are better), at most `most` steps; and the launch,
+// with the source amplitude of each step.
+constexpr int kSmallSteps = 8;
+struct SmallPlan {
+  int tw = 0, th = 0, steps = 0;
+  double us = 1e300;                  // estimated time per step
+};
+SmallPlan cart2d_small_plan(const CartGeom &g, const CartStepArgs &a, bool fp64, int64_t most);
+cudaError_t launch_cart2d_small(const CartGeom &g, const CartStepArgs &a, const SmallPlan &pl,
+                                const double *amp, bool fp64, cudaStream_t st);
 // FP32 3-D step with tau = 0 where the side-split kernel would run (gks_cart3d_tau0.cu).
 bool cart3d_tau0_supported(const CartGeom &g, const CartStepArgs &a);
 cudaError_t launch_cart3d_tau0(const CartGeom &g, const CartStepArgs &a, cudaStream_t st);

@@ -5,7 +5,7 @@ import numpy as np
 import pytest
 
 from paper_2412_16845_gb300 import workloads as wl
-from paper_2412_16845_gb300.gks import GKSSolver
+from paper_2412_16845_gb300.gks import GKSSolver, gks_step_window
 from tests.oracle_runs import oracle_cart_run, rel_l2
 
 pytestmark = pytest.mark.gpu
@@ -35,9 +35,13 @@ def _grid(n, bc, seed, source=True, limiter=None, stretch=1.2):
                            src=(1.0, 20.0, 0.02, 0.02), c_lattice=0.0, limiter=limiter)
 
 
-def _check(w, precision, steps):
+def _check(w, precision, steps, march=False):
+    """march: windowed steps over the whole grid, which small grids do not take several at a time."""
     s = GKSSolver.from_workload(w, precision=precision)
-    s.step(steps)
+    if march:
+        gks_step_window(s.ctx, steps, 0, w.n[0], 0, w.n[1])
+    else:
+        s.step(steps)
     out = s.read_fields()
     c = s.info()["c"]
     s.close()
@@ -54,13 +58,25 @@ def _check(w, precision, steps):
 ])
 def test_2d_tiles(n, bc, precision):
     sides = tuple({"n": "nrbc", "p": "periodic", "m": "pec"}[b] for b in bc)
-    _check(_grid(n, sides, seed=n[0] + 7 * n[1]), precision, 9)
+    _check(_grid(n, sides, seed=n[0] + 7 * n[1]), precision, 9, march=True)
 
 
 @pytest.mark.parametrize("precision", ["fp32", "fp64"])
 @pytest.mark.parametrize("n,bc", [((63, 9), "nrbc"), ((250, 6), "periodic"), ((130, 17), "pec")])
 def test_2d_limited_tiles(n, bc, precision):
-    _check(_grid(n, (bc,) * 4, seed=n[0], limiter="vanleer"), precision, 9)
+    _check(_grid(n, (bc,) * 4, seed=n[0], limiter="vanleer"), precision, 9, march=True)
+
+
+# several steps per launch on small grids: tiles of 4 to 24 cells, 1 to 8 steps, walls inside a margin
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("n,bc,steps,limiter", [
+    ((64, 64), "pppp", 19, None), ((100, 100), "nnnn", 23, None), ((41, 77), "mmnn", 8, None),
+    ((5, 3), "nmpp", 11, None), ((1, 1), "nnnn", 3, None), ((2, 2), "mmmm", 7, None),
+    ((17, 90), "ppmn", 1, None), ((33, 20), "nnmm", 9, "vanleer"), ((3, 50), "pppp", 16, "vanleer"),
+])
+def test_2d_small_grids(n, bc, steps, limiter, precision):
+    sides = tuple({"n": "nrbc", "p": "periodic", "m": "pec"}[b] for b in bc)
+    _check(_grid(n, sides, seed=n[0] + 3 * n[1], limiter=limiter), precision, steps)
 
 
 def test_2d_extreme_permittivity_keeps_its_results():
