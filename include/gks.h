@@ -170,6 +170,14 @@ gks_status gks_step(gks_ctx *ctx, int64_t n_steps);
 gks_status gks_step_window(gks_ctx *ctx, int64_t n_steps, int64_t x0, int64_t x1, int64_t y0,
                            int64_t y1);
 
+/* Enqueue one step from the state src into dst (device, gks_state_layout bytes each, distinct) over
+ * the window [x0, x1) x [y0, y1) of a 2-D Cartesian grid, as step number `step` (the source is taken
+ * at t0 + step dt).  The context's own state, time and step counter stay.  Entries of dst outside the
+ * window are left as they are or hold stale values; the window's cells need src on the window
+ * widened by two cells.  Asynchronous. */
+gks_status gks_step_state_window(gks_ctx *ctx, const void *src, void *dst, int64_t step, int64_t x0,
+                                 int64_t x1, int64_t y0, int64_t y1);
+
 /* Wait for the stream, then copy the fields to out ([ncomp][n_cells] doubles, user order,
  * host).  GKS_E_NONFINITE if a step produced a non-finite value, GKS_E_TIMEOUT if a staged
  * kernel's bounded wait for its tensor copies ran out. */
@@ -230,6 +238,15 @@ gks_status gks_adjoint_seed(gks_ctx *ctx, const void *state, void *adj);
 gks_status gks_adjoint_step(gks_ctx *ctx, const void *state_n, const void *state_np1,
                             const void *adj_in, void *adj_out, double *grad_eps,
                             int32_t add_probe);
+
+/* gks_adjoint_step computing lambda^n only on the window [x0, x1) x [y0, y1) (adj_out elsewhere stays
+ * or holds stale values) and the eps-gradient of the design cells in it.  For windows outside which
+ * lambda^n is zero or not needed: it is zero beyond two cells per step around the probe, and only the
+ * cells within two cells per remaining step of the design region act on the gradient.  adj_in must
+ * hold lambda^{n+1} on the window widened by two cells. */
+gks_status gks_adjoint_step_window(gks_ctx *ctx, const void *state_n, const void *state_np1,
+                                   const void *adj_in, void *adj_out, double *grad_eps,
+                                   int32_t add_probe, int64_t x0, int64_t x1, int64_t y0, int64_t y1);
 
 /* ---- Domain split across ranks (one process per GPU).  The finite-volume update of Sec. 3.1
  * reaches two cells along every axis (the Green-Gauss gradient of Sec. 3.1, then the face flux

@@ -14,9 +14,9 @@ import math
 
 import numpy as np
 
-from .gks import (GKSSolver, gks_adjoint_seed, gks_adjoint_step, gks_copy_state,
-                  gks_copy_state_box, gks_load_state, gks_objective, gks_reset_objective,
-                  gks_set_materials_box, gks_set_objective, gks_state_layout, gks_step_window)
+from .gks import (GKSSolver, gks_adjoint_seed, gks_adjoint_step_window, gks_copy_state,
+                  gks_load_state, gks_objective, gks_reset_objective, gks_set_materials_box,
+                  gks_set_objective, gks_state_layout, gks_step_state_window)
 
 
 def design_box(design, nx):
@@ -63,29 +63,44 @@ class DesignProblem:
         self.final = None
         self.eps_design = None
         # the adjoint reads states only on the design cells and their two-cell stencil and on
-        # the probe: that box (cbox) is what is stored of a recomputed state.  Step m of a
-        # segment of k steps is recomputed on cbox widened by 2 (k - m) cells, its domain of
-        # dependence, so the window shrinks by the stencil radius every step.
+        # the probe: cbox.  Step m of a segment of k steps is recomputed on cbox widened by
+        # 2 (k - m) cells, its domain of dependence, so the window shrinks by the stencil radius
+        # every step.
         nx, ny = w.n
         self.nx, self.ny = nx, ny
         self.per = (w.bc[0] == "periodic", w.bc[2] == "periodic")
-        cells = np.concatenate([self.design, np.asarray(w.probe, dtype=np.int64)])
-        xs, ys = cells % nx, cells // nx
-        self.cbox = (max(0, int(xs.min()) - 2), min(nx, int(xs.max()) + 3),
-                     max(0, int(ys.min()) - 2), min(ny, int(ys.max()) + 3))
+        self.pbox = self._box(w.probe)
+        self.cbox = self._widen(self._box(np.concatenate([self.design,
+                                                          np.asarray(w.probe, dtype=np.int64)])), 2)
 
-    def _window(self, r):
-        """cbox widened by r cells, clipped to the grid (a whole periodic axis once it wraps)."""
-        x0, x1, y0, y1 = self.cbox
-        x0, x1, y0, y1 = x0 - r, x1 + r, y0 - r, y1 + r
+    def _box(self, cells):
+        """Half-open bounding box (x0, x1, y0, y1) of cells."""
+        xs, ys = np.asarray(cells) % self.nx, np.asarray(cells) // self.nx
+        return int(xs.min()), int(xs.max()) + 1, int(ys.min()), int(ys.max()) + 1
+
+    def _widen(self, box, r):
+        """box widened by r cells, clipped to the grid (a whole periodic axis once it wraps)."""
+        x0, x1, y0, y1 = box[0] - r, box[1] + r, box[2] - r, box[3] + r
         if x0 < 0 or x1 > self.nx:
             x0, x1 = (0, self.nx) if self.per[0] else (max(0, x0), min(self.nx, x1))
         if y0 < 0 or y1 > self.ny:
             y0, y1 = (0, self.ny) if self.per[1] else (max(0, y0), min(self.ny, y1))
         return x0, x1, y0, y1
 
+    def _lambda_window(self, n):
+        """Where lambda^n is computed, or None: it is zero beyond two cells per step n .. N around the
+        probe, and the steps below n carry only the cells within 2 n of the design region into the
+        gradient."""
+        a = self._widen(self.pbox, 2 * (self.N - n))
+        b = self._widen(self.dbox, 2 * n + 2)
+        x0, x1, y0, y1 = max(a[0], b[0]), min(a[1], b[1]), max(a[2], b[2]), min(a[3], b[3])
+        return (x0, x1, y0, y1) if x0 < x1 and y0 < y1 else None
+
     def _buf(self):
         return self.torch.empty(self.elems, dtype=self.dtype, device="cuda")
+
+    def _zeros(self):
+        return self.torch.zeros(self.elems, dtype=self.dtype, device="cuda")
 
     def set_design(self, eps_design):
         e = np.array(eps_design, dtype=np.float64).reshape(-1)
@@ -127,29 +142,30 @@ class DesignProblem:
         torch = self.torch
         if self.checkpoints is None:
             raise RuntimeError("forward() with keep_checkpoints=True must come first")
-        lam = self._buf()
-        lam2 = self._buf()
+        # (zero where lambda is never computed; the pool's entries off the recomputed windows are
+        # never read into a result, but have to be finite)
+        lam, lam2 = self._zeros(), self._zeros()
         grad = torch.zeros(self.design.size, dtype=torch.float64, device="cuda")
         gks_adjoint_seed(self.ctx, self.final.data_ptr(), lam.data_ptr())
-        # the recomputed states of one segment live in K buffers reused by every segment
-        # (addresses, windows and the box taken once, not per step)
-        pool = [self._buf() for _ in range(self.K)]
+        # the recomputed states of one segment live in K buffers reused by every segment, each step
+        # written straight from one into the next (addresses taken once, not per step)
+        pool = [self._zeros() for _ in range(self.K)]
         pool_ptr = [b.data_ptr() for b in pool]
         lam_ptr, lam2_ptr, grad_ptr = lam.data_ptr(), lam2.data_ptr(), grad.data_ptr()
-        ctx, cbox = self.ctx, self.cbox
+        ctx = self.ctx
+        windows = [self._widen(self.cbox, 2 * r) for r in range(self.K)]
         for (s, ckb), e in zip(reversed(self.checkpoints),
                                reversed([c[0] for c in self.checkpoints[1:]] + [self.N])):
             k = e - s
             # recompute V^s .. V^e of this segment
-            ck_ptr = ckb.data_ptr()
-            gks_load_state(ctx, ck_ptr, s)
-            ptrs = [ck_ptr] + pool_ptr[:k]
+            ptrs = [ckb.data_ptr()] + pool_ptr[:k]
             for m in range(1, k + 1):
-                gks_step_window(ctx, 1, *self._window(2 * (k - m)))
-                gks_copy_state_box(ctx, ptrs[m], *cbox)
+                gks_step_state_window(ctx, ptrs[m - 1], ptrs[m], s + m - 1, *windows[k - m])
             for n in range(e - 1, s - 1, -1):
-                gks_adjoint_step(ctx, ptrs[n - s], ptrs[n - s + 1], lam_ptr, lam2_ptr, grad_ptr,
-                                 n >= 1)
+                win = self._lambda_window(n)
+                if win is not None:
+                    gks_adjoint_step_window(ctx, ptrs[n - s], ptrs[n - s + 1], lam_ptr, lam2_ptr,
+                                            grad_ptr, n >= 1, *win)
                 lam_ptr, lam2_ptr = lam2_ptr, lam_ptr
         del pool
         return grad

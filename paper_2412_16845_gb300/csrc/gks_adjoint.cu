@@ -128,6 +128,7 @@ struct AdjArgs {
   int64_t pitch, cstride;
   int perx, pery;
   FaceK<T> fx, fy;
+  int wx0, wx1, wy0, wy1;         // lambda^n cells to compute (half open)
 };
 
 __device__ __forceinline__ int wc(int i, int n, int periodic) {
@@ -253,12 +254,12 @@ __global__ void __launch_bounds__(AWARPS * 32) adjoint_lambda_kernel(const AdjAr
   const int lane = threadIdx.x & 31;
   const int wid = blockIdx.x * AWARPS + (threadIdx.x >> 5);
   const int strip = wid % nstrips, chunk = wid / nstrips;
-  const int y0 = chunk * rows;
-  if (y0 >= p.ny) return;                              // whole warp leaves together
-  const int y1 = min(y0 + rows, p.ny);
-  const int x0 = strip * AWCOLS;
+  const int y0 = p.wy0 + chunk * rows;
+  if (y0 >= p.wy1) return;                             // whole warp leaves together
+  const int y1 = min(y0 + rows, p.wy1);
+  const int x0 = p.wx0 + strip * AWCOLS;
   const int X = x0 - 2 + 2 * lane;
-  const int xend = min(x0 + AWCOLS, p.nx);
+  const int xend = min(x0 + AWCOLS, p.wx1);
   // D_x^T weights of the lane's two columns (cell i gets cl dbar_{i-1} - cr dbar_{i+1} +
   // cs dbar_i: d_i = V(i+1) - V(i-1) with clamped ends, or wrapped)
   T cl[2], cr[2], cs[2];
@@ -444,13 +445,14 @@ __global__ void __launch_bounds__(GX * GY) adjoint_post_kernel(const AdjArgs<T> 
   const int tx = tid % GX, ty = tid / GX;
   const int gx = x0 + tx, gy = y0 + ty;
   const int64_t o = (int64_t)gy * p.pitch + gx;
-  if (p.pw && gx >= p.px0 && gx < p.px1 && gy >= p.py0 && gy < p.py1) {
+  if (p.pw && gx < p.wx1 && gy < p.wy1 && gx >= p.px0 && gx < p.px1 && gy >= p.py0 && gy < p.py1) {
     const double w = p.pw[(int64_t)(gy - p.py0) * (p.px1 - p.px0) + (gx - p.px0)];
     p.lout[o] += T(p.dt2 * w) * p.Vn[o];
   }
   if (!p.grad) return;                                  // uniform over the launch
   // the cell's own loads go out before the staging so that their latencies overlap
-  const bool in_box = gx >= p.dx0 && gx < p.dx1 && gy >= p.dy0 && gy < p.dy1;
+  const bool in_box = gx >= p.dx0 && gx < p.dx1 && gy >= p.dy0 && gy < p.dy1 && gx < p.wx1 &&
+                      gy < p.wy1;
   const int slot = in_box ? p.dslot[o] : -1;
   const T en1 = slot >= 0 ? p.Vn1[o] : T(0);
   const double g_old = slot >= 0 ? p.grad[slot] : 0.0;
@@ -513,7 +515,7 @@ __global__ void probe_grad_kernel(const T *__restrict__ V, T *__restrict__ lam,
 }
 
 // q(V) = dt sum_P |Omega| Ez^2, deterministic: block b sums its contiguous slice of the probe
-// list in a fixed tree order into part[b]; the last block to finish (ticket) adds the partials
+// list in a fixed order into part[b]; the last block to finish (ticket) adds the partials
 // in index order and folds dt * sum into the Kahan-compensated running sum acc = (sum, comp).
 constexpr int OBJ_T = 256;
 
@@ -522,7 +524,7 @@ __global__ void __launch_bounds__(OBJ_T) objective_kernel(const T *__restrict__ 
                                                           const int64_t *__restrict__ off,
                                                           const double *__restrict__ w, int64_t np,
                                                           double dt, double *__restrict__ acc) {
-  __shared__ double red[OBJ_T];
+  __shared__ double red[OBJ_T / 32];
   __shared__ int last;
   double *part = acc + 2;
   unsigned *ticket = reinterpret_cast<unsigned *>(acc + 2 + kObjParts);
@@ -533,14 +535,14 @@ __global__ void __launch_bounds__(OBJ_T) objective_kernel(const T *__restrict__ 
     const double e = double(V[off[i]]);
     a += w[i] * e * e;
   }
-  red[threadIdx.x] = a;
+  // fixed tree: lanes, then the warps' sums in order (a barrier per level of a shared-memory tree
+  // was most of this latency-bound kernel)
+  for (int s = 16; s > 0; s >>= 1) a += __shfl_down_sync(0xffffffffu, a, s);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = a;
   __syncthreads();
-  for (int s = OBJ_T / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
-    __syncthreads();
-  }
   if (threadIdx.x == 0) {
-    part[blockIdx.x] = red[0];
+    for (int i = 1; i < OBJ_T / 32; ++i) a += red[i];
+    part[blockIdx.x] = a;
     __threadfence();
     last = atomicAdd(ticket, 1u) == gridDim.x - 1;
   }
@@ -580,6 +582,9 @@ cudaError_t adjoint_t(const CartGeom &g, const AdjointArgs &a, cudaStream_t st) 
   p.perx = g.periodic[0]; p.pery = g.periodic[1];
   p.fx = make_face_k<T>(a.C, g.h[0], g.h[1], a.c, 1.0, 1.0);
   p.fy = make_face_k<T>(a.C, g.h[1], g.h[0], a.c, -1.0, -1.0);
+  // pairs are loaded and stored as 8- or 16-byte words: the window starts on an even column
+  p.wx0 = a.window[0] & ~1; p.wx1 = a.window[1]; p.wy0 = a.window[2]; p.wy1 = a.window[3];
+  const bool tau0 = adjoint_tau0_supported(g, a);
   // strips of 60 columns; rows per warp chosen so that the warps fit in one wave
   static int resident = 0;   // warps of this kernel resident on the GPU at once
   if (!resident) {
@@ -589,19 +594,25 @@ cudaError_t adjoint_t(const CartGeom &g, const AdjointArgs &a, cudaStream_t st) 
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, adjoint_lambda_kernel<T>, AWARPS * 32, 0);
     resident = sms * (bps > 0 ? bps : 1) * AWARPS;
   }
-  const int nstrips = (g.nx + AWCOLS - 1) / AWCOLS;
-  int rows = g.ny;
+  const int wrows = p.wy1 - p.wy0;
+  const int nstrips = (p.wx1 - p.wx0 + AWCOLS - 1) / AWCOLS;
+  int rows = wrows;
   const int target = resident;
   if (nstrips < target) {
     const int chunks = (target + nstrips - 1) / nstrips;
-    rows = (g.ny + chunks - 1) / chunks;
+    rows = (wrows + chunks - 1) / chunks;
   }
   rows = rows < 16 ? 16 : (rows > 256 ? 256 : rows);
-  const int nchunks = (g.ny + rows - 1) / rows;
+  const int nchunks = (wrows + rows - 1) / rows;
   const int64_t nwarps = (int64_t)nstrips * nchunks;
   const int grid = (int)((nwarps + AWARPS - 1) / AWARPS);
-  adjoint_lambda_kernel<T><<<grid, AWARPS * 32, 0, st>>>(p, nstrips, rows);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e;
+  if (tau0 && sizeof(T) == 4) {
+    e = launch_adjoint_tau0(g, a, st);
+  } else {
+    adjoint_lambda_kernel<T><<<grid, AWARPS * 32, 0, st>>>(p, nstrips, rows);
+    e = cudaGetLastError();
+  }
   if (e != cudaSuccess) return e;
   // probe term and eps-gradient over the bounding box of the probe and the design cells
   if (p.grad && (p.dx1 <= p.dx0 || p.dy1 <= p.dy0)) p.grad = nullptr;
@@ -612,6 +623,11 @@ cudaError_t adjoint_t(const CartGeom &g, const AdjointArgs &a, cudaStream_t st) 
     b[0] = std::min(b[0], p.px0); b[1] = std::max(b[1], p.px1);
     b[2] = std::min(b[2], p.py0); b[3] = std::max(b[3], p.py1);
   }
+  // (lambda^{n+1} is zero near any design cell outside the window)
+  b[0] = std::max(b[0], a.window[0]); b[1] = std::min(b[1], a.window[1]);
+  b[2] = std::max(b[2], a.window[2]); b[3] = std::min(b[3], a.window[3]);
+  if (b[0] >= b[1] || b[2] >= b[3]) return cudaSuccess;
+  if (tau0) return launch_adjoint_post_tau0(g, a, b, sizeof(T) == 8, st);
   dim3 gg((b[1] - b[0] + GX - 1) / GX, (b[3] - b[2] + GY - 1) / GY);
   adjoint_post_kernel<T><<<gg, GX * GY, 0, st>>>(p, b[0], b[2]);
   return cudaGetLastError();

@@ -587,8 +587,18 @@ gks_status gks_set_dt(gks_ctx *ctx, double dt) {
 
 namespace {
 
-// Advance n_steps over the window [x0, x1) x [y0, y1) (2-D) or the whole mesh.
-gks_status step_impl(gks_ctx *ctx, int64_t n_steps, const int win[4], bool objective) {
+// dt times the source's waveform at step `step`.
+double source_amplitude(const gks_ctx *ctx, int64_t step) {
+  if (!ctx->src) return 0.0;
+  const double t = ctx->t0 + (double)step * ctx->dt, tt = t - ctx->srcT0;
+  if (ctx->srcKind == 1)
+    return tt >= 0.0 ? ctx->dt * ctx->srcA * std::cos(2.0 * M_PI * ctx->srcF0 * tt) : 0.0;
+  return ctx->dt * ctx->srcA * std::exp(-(tt / ctx->srcS) * (tt / ctx->srcS)) *
+         std::sin(2.0 * M_PI * ctx->srcF0 * tt);
+}
+
+// The arguments every step of the context over the window [x0, x1) x [y0, y1) shares.
+gks::CartStepArgs step_args(const gks_ctx *ctx, const int win[4]) {
   gks::CartStepArgs a;
   a.eps = ctx->eps;
   a.mu = ctx->mu;
@@ -600,22 +610,19 @@ gks_status step_impl(gks_ctx *ctx, int64_t n_steps, const int win[4], bool objec
   a.flag = ctx->flag;
   a.limiter = ctx->limiter;
   a.eps_normal = ctx->eps_normal;
-  // dt times the source's waveform at step `step`
-  auto amplitude = [ctx](int64_t step) {
-    if (!ctx->src) return 0.0;
-    const double t = ctx->t0 + (double)step * ctx->dt, tt = t - ctx->srcT0;
-    if (ctx->srcKind == 1)
-      return tt >= 0.0 ? ctx->dt * ctx->srcA * std::cos(2.0 * M_PI * ctx->srcF0 * tt) : 0.0;
-    return ctx->dt * ctx->srcA * std::exp(-(tt / ctx->srcS) * (tt / ctx->srcS)) *
-           std::sin(2.0 * M_PI * ctx->srcF0 * tt);
-  };
+  return a;
+}
+
+// Advance n_steps over the window [x0, x1) x [y0, y1) (2-D) or the whole mesh.
+gks_status step_impl(gks_ctx *ctx, int64_t n_steps, const int win[4], bool objective) {
+  gks::CartStepArgs a = step_args(ctx, win);
   // windowed steps (objective = false) march: their windows are recomputed step by step
   const bool small = objective && ctx->kind == GKS_CARTESIAN && ctx->dim == 2 && !ctx->phm;
   const bool probe = objective && ctx->np > 0;       // needs the state after every step
   gks::SmallPlan pl;
   if (small) pl = gks::cart2d_small_plan(ctx->g, a, ctx->fp64, probe ? 1 : n_steps);
   for (int64_t n = 0; n < n_steps;) {
-    a.src_amp = amplitude(ctx->step);
+    a.src_amp = source_amplitude(ctx, ctx->step);
     a.V = ctx->V[ctx->cur];
     a.Vout = ctx->V[ctx->cur ^ 1];
     cudaError_t e;
@@ -625,7 +632,7 @@ gks_status step_impl(gks_ctx *ctx, int64_t n_steps, const int win[4], bool objec
     if (pl.steps > 0) {
       double amp[gks::kSmallSteps];
       done = pl.steps;
-      for (int s = 0; s < done; ++s) amp[s] = amplitude(ctx->step + s);
+      for (int s = 0; s < done; ++s) amp[s] = source_amplitude(ctx, ctx->step + s);
       e = gks::launch_cart2d_small(ctx->g, a, pl, amp, ctx->fp64, ctx->st);
       ctx->launches += 1;
     } else if (ctx->kind == GKS_TET) {
@@ -677,6 +684,25 @@ gks_status gks_step_window(gks_ctx *ctx, int64_t n_steps, int64_t x0, int64_t x1
   if (!ctx->fields_written) return fail(ctx, GKS_E_STATE, "gks_write_fields must come first");
   const int win[4] = {(int)x0, (int)x1, (int)y0, (int)y1};
   return step_impl(ctx, n_steps, win, false);
+}
+
+gks_status gks_step_state_window(gks_ctx *ctx, const void *src, void *dst, int64_t step, int64_t x0,
+                                 int64_t x1, int64_t y0, int64_t y1) {
+  if (!ctx) return GKS_E_ARG;
+  if (ctx->kind != GKS_CARTESIAN || ctx->dim != 2)
+    return fail(ctx, GKS_E_UNSUPPORTED, "windowed steps need a 2-D Cartesian grid");
+  if (ctx->phm) return fail(ctx, GKS_E_UNSUPPORTED, "windowed steps do not cover divergence cleaning");
+  if (!src || !dst || src == dst || step < 0) return fail(ctx, GKS_E_ARG, "src / dst / step");
+  if (x0 < 0 || y0 < 0 || x1 > ctx->g.nx || y1 > ctx->g.ny || x0 >= x1 || y0 >= y1)
+    return fail(ctx, GKS_E_ARG, "window outside the grid or empty");
+  const int win[4] = {(int)x0, (int)x1, (int)y0, (int)y1};
+  gks::CartStepArgs a = step_args(ctx, win);
+  a.V = src;
+  a.Vout = dst;
+  a.src_amp = source_amplitude(ctx, step);
+  GKS_CUDA(gks::launch_cart2d_step(ctx->g, a, ctx->fp64, ctx->st));
+  ctx->launches += 1;
+  return GKS_OK;
 }
 
 gks_status gks_copy_state_box(gks_ctx *ctx, void *dst, int64_t x0, int64_t x1, int64_t y0,
@@ -856,6 +882,13 @@ gks_status gks_adjoint_seed(gks_ctx *ctx, const void *state, void *adj) {
 gks_status gks_adjoint_step(gks_ctx *ctx, const void *state_n, const void *state_np1,
                             const void *adj_in, void *adj_out, double *grad_eps,
                             int32_t add_probe) {
+  return gks_adjoint_step_window(ctx, state_n, state_np1, adj_in, adj_out, grad_eps, add_probe, 0,
+                                 ctx ? ctx->g.nx : 0, 0, ctx ? ctx->g.ny : 0);
+}
+
+gks_status gks_adjoint_step_window(gks_ctx *ctx, const void *state_n, const void *state_np1,
+                                   const void *adj_in, void *adj_out, double *grad_eps,
+                                   int32_t add_probe, int64_t x0, int64_t x1, int64_t y0, int64_t y1) {
   if (!ctx) return GKS_E_ARG;
   if (ctx->kind != GKS_CARTESIAN || ctx->dim != 2)
     return fail(ctx, GKS_E_UNSUPPORTED, "the adjoint needs a 2-D Cartesian grid");
@@ -872,7 +905,12 @@ gks_status gks_adjoint_step(gks_ctx *ctx, const void *state_n, const void *state
   if (ctx->nd > 0 && (!grad_eps || !state_n || !state_np1))
     return fail(ctx, GKS_E_ARG, "the eps-gradient needs both states and grad_eps");
   if (add_probe && ctx->np > 0 && !state_n) return fail(ctx, GKS_E_ARG, "state_n is NULL");
+  if (x0 < 0 || y0 < 0 || x1 > ctx->g.nx || y1 > ctx->g.ny || x0 >= x1 || y0 >= y1)
+    return fail(ctx, GKS_E_ARG, "window outside the grid or empty");
   gks::AdjointArgs a;
+  a.window[0] = (int)x0; a.window[1] = (int)x1; a.window[2] = (int)y0; a.window[3] = (int)y1;
+  a.eps_normal = ctx->eps_normal;
+  a.flag = ctx->flag;
   a.lam_in = adj_in;
   a.lam_out = adj_out;
   a.eps = ctx->eps;

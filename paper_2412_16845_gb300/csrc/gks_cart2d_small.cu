@@ -19,6 +19,7 @@
 #include "gks_flux2.cuh"
 #include "gks_internal.h"
 #include "gks_rcp.cuh"
+#include "gks_tau0_2d.cuh"
 
 namespace gks {
 namespace {
@@ -27,21 +28,6 @@ template <typename T>
 constexpr int NT = sizeof(T) == 4 ? 512 : 256;   // threads per CTA
 constexpr int kMaxSteps = kSmallSteps;
 constexpr int NF = 22;                // values a cell of the region keeps in shared memory
-
-template <typename T>
-struct AxisS {
-  T ic, mq, m4, c0, l4, ka, kE, sE, sH;
-};
-
-template <typename T>
-AxisS<T> make_axis_s(const double C[5], double c, double hn, double ht, double sign) {
-  const double ic = sign / c, k3 = sign * C[2] / (2.0 * hn * C[0]);
-  AxisS<T> k;
-  k.ic = T(ic); k.mq = T(-0.25 * ic); k.m4 = T(-4.0 * ic); k.c0 = T(k3 - 0.25 * ic);
-  k.l4 = T(-4.0 * k3 * ic); k.ka = T(-sign * C[2] / (2.0 * ht * C[0])); k.kE = T(2.0 * k3);
-  k.sE = T(-sign * 0.5 * C[0] / hn); k.sH = T(-sign * C[0] / hn);
-  return k;
-}
 
 template <typename T>
 struct SmallArgs {
@@ -53,7 +39,7 @@ struct SmallArgs {
   int nx, ny;
   int64_t pitch, cstride;
   int perx, pery, pec[4];
-  AxisS<T> X, Y;
+  AxisK<T> X, Y;
   int *flag;
   int tw, th, steps, tiles_x;         // tile, steps of this launch, tiles along x
 };
@@ -151,7 +137,7 @@ __global__ void __launch_bounds__(NT<T>) cart2d_small_kernel(const __grid_consta
       const T bx = raw_slope<LIMIT>(fb[i - 1], b, fb[i + 1]), ay = raw_slope<LIMIT>(fa[i - RW], a, fa[i + RW]);
       const T ue = k * e, ux = k * ex, uy = k * ey;
       const bool gxz = (nxl && x < 0) || (nxh && x >= p.nx), gyz = (nyl && y < 0) || (nyh && y >= p.ny);
-      auto sides = [&](const AxisS<T> &K, T bb, T en, T bn, T un, T at, bool zero, T *lo, T *hi) {
+      auto sides = [&](const AxisK<T> &K, T bb, T en, T bn, T un, T at, bool zero, T *lo, T *hi) {
         const T ev = mad(K.mq, en, bb), od = mad(K.m4, e, bn);
         const T eq = mad(K.ka, at, mad(K.c0, bn, ue)), oq = mad(K.l4, en, mad(K.m4, bb, un));
         hi[i] = zero ? T(0) : mad(T(0.25), od, ev);
@@ -257,8 +243,8 @@ cudaError_t launch_t(const CartGeom &g, const CartStepArgs &a, const SmallPlan &
   p.pitch = g.pitch; p.cstride = g.cstride;
   p.perx = g.periodic[0]; p.pery = g.periodic[1];
   for (int k = 0; k < 4; ++k) p.pec[k] = g.pec[k];
-  p.X = make_axis_s<T>(a.C, a.c, g.h[0], g.h[1], 1.0);
-  p.Y = make_axis_s<T>(a.C, a.c, g.h[1], g.h[0], -1.0);
+  p.X = make_axis<T>(a.C, a.c, g.h[0], g.h[1], 1.0);
+  p.Y = make_axis<T>(a.C, a.c, g.h[1], g.h[0], -1.0);
   p.flag = a.flag;
   p.tw = pl.tw; p.th = pl.th; p.steps = pl.steps;
   p.tiles_x = (g.nx + pl.tw - 1) / pl.tw;

@@ -118,7 +118,16 @@ struct AdjointArgs {
   double dt;
   double C[5];
   double c;
+  int window[4];            // x0, x1, y0, y1 (half open) of the cells of lambda^n to compute
+  bool eps_normal;          // as CartStepArgs
+  int *flag;
 };
+// lambda march (FP32) and probe term / eps-gradient for tau = 0 (gks_adjoint_tau0.cu); `box` covers the
+// probe and design cells of the window.
+bool adjoint_tau0_supported(const CartGeom &g, const AdjointArgs &a);
+cudaError_t launch_adjoint_tau0(const CartGeom &g, const AdjointArgs &a, cudaStream_t st);
+cudaError_t launch_adjoint_post_tau0(const CartGeom &g, const AdjointArgs &a, const int box[4],
+                                     bool fp64, cudaStream_t st);
 cudaError_t launch_adjoint_step(const CartGeom &g, const AdjointArgs &a, bool fp64,
                                 cudaStream_t st);
 cudaError_t launch_probe_grad(const void *V, void *lam, const int64_t *off, const double *w,

@@ -94,6 +94,13 @@ SIGNATURES = {
     "gks_adjoint_seed": (ctypes.c_int, [_CTX, ctypes.c_void_p, ctypes.c_void_p]),
     "gks_adjoint_step": (ctypes.c_int, [_CTX, ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
                                         ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32]),
+    "gks_adjoint_step_window": (ctypes.c_int, [_CTX, ctypes.c_void_p, ctypes.c_void_p,
+                                               ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
+                                               ctypes.c_int32, ctypes.c_int64, ctypes.c_int64,
+                                               ctypes.c_int64, ctypes.c_int64]),
+    "gks_step_state_window": (ctypes.c_int, [_CTX, ctypes.c_void_p, ctypes.c_void_p,
+                                             ctypes.c_int64, ctypes.c_int64, ctypes.c_int64,
+                                             ctypes.c_int64, ctypes.c_int64]),
     "gks_energy_noalloc": (ctypes.c_int, [ctypes.c_int32, ctypes.c_int32, ctypes.c_int64,
                                           ctypes.c_double, ctypes.c_void_p, ctypes.c_void_p,
                                           ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p]),
@@ -280,6 +287,17 @@ def gks_adjoint_seed(ctx, state_ptr, adj_ptr):
 def gks_adjoint_step(ctx, state_n, state_np1, adj_in, adj_out, grad_eps, add_probe):
     _check(ctx, load_library().gks_adjoint_step(ctx, state_n, state_np1, adj_in, adj_out,
                                                 grad_eps, 1 if add_probe else 0))
+
+
+def gks_adjoint_step_window(ctx, state_n, state_np1, adj_in, adj_out, grad_eps, add_probe, x0, x1,
+                            y0, y1):
+    _check(ctx, load_library().gks_adjoint_step_window(ctx, state_n, state_np1, adj_in, adj_out,
+                                                       grad_eps, 1 if add_probe else 0, x0, x1, y0,
+                                                       y1))
+
+
+def gks_step_state_window(ctx, src, dst, step, x0, x1, y0, y1):
+    _check(ctx, load_library().gks_step_state_window(ctx, src, dst, step, x0, x1, y0, y1))
 
 
 def gks_sync(ctx):
