@@ -18,6 +18,7 @@
 
 #include "gks_flux2.cuh"
 #include "gks_internal.h"
+#include "gks_pdl.cuh"
 
 namespace gks {
 namespace {
@@ -520,10 +521,11 @@ __global__ void probe_grad_kernel(const T *__restrict__ V, T *__restrict__ lam,
 constexpr int OBJ_T = 256;
 
 template <typename T>
-__global__ void __launch_bounds__(OBJ_T) objective_kernel(const T *__restrict__ V,
-                                                          const int64_t *__restrict__ off,
-                                                          const double *__restrict__ w, int64_t np,
-                                                          double dt, double *__restrict__ acc) {
+__global__ void __launch_bounds__(OBJ_T) objective_kernel(const T *V, const int64_t *off,
+                                                          const double *w, int64_t np, double dt,
+                                                          double *acc) {
+  grid_wait();
+  grid_trigger();
   __shared__ double red[OBJ_T / 32];
   __shared__ int last;
   double *part = acc + 2;
@@ -659,13 +661,10 @@ cudaError_t launch_objective(const void *V, const int64_t *off, const double *w,
                              double dt, double *acc, bool fp64, cudaStream_t st) {
   if (np <= 0) return cudaSuccess;
   const int blocks = (int)std::min<int64_t>(kObjParts, (np + OBJ_T - 1) / OBJ_T);
-  if (fp64)
-    objective_kernel<double><<<blocks, OBJ_T, 0, st>>>(static_cast<const double *>(V), off, w, np,
-                                                       dt, acc);
-  else
-    objective_kernel<float><<<blocks, OBJ_T, 0, st>>>(static_cast<const float *>(V), off, w, np,
-                                                      dt, acc);
-  return cudaGetLastError();
+  return fp64 ? launch_pdl(objective_kernel<double>, blocks, OBJ_T, 0, st,
+                           static_cast<const double *>(V), off, w, np, dt, acc)
+              : launch_pdl(objective_kernel<float>, blocks, OBJ_T, 0, st,
+                           static_cast<const float *>(V), off, w, np, dt, acc);
 }
 
 }  // namespace gks

@@ -22,6 +22,7 @@
 #include <type_traits>
 
 #include "gks_internal.h"
+#include "gks_pdl.cuh"
 #include "gks_rcp.cuh"
 #include "gks_tau0_2d.cuh"
 #include "gks_tma.cuh"
@@ -61,9 +62,9 @@ struct Axis {                           // AxisK with the quarters of the transp
 };
 
 struct Args {
-  float *__restrict__ out;
-  const float *__restrict__ lam;
-  const float *__restrict__ eps;
+  float *out;                           // (not __restrict__: gks_pdl.cuh)
+  const float *lam;
+  const float *eps;
   int nx, ny;
   int64_t pitch, cstride;
   int perx, pery;
@@ -102,6 +103,8 @@ __global__ void __launch_bounds__(WARPS * 32, 5)
     adjoint_tau0_kernel(const __grid_constant__ CUtensorMap tmL, const __grid_constant__ CUtensorMap tmE,
                         const __grid_constant__ Args p) {
   extern __shared__ __align__(128) unsigned char smem_a[];
+  grid_wait();
+  grid_trigger();
   Stage &s = *reinterpret_cast<Stage *>(smem_a);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int tile = blockIdx.x % p.ntiles, chunk = blockIdx.x / p.ntiles;
@@ -153,7 +156,7 @@ __global__ void __launch_bounds__(WARPS * 32, 5)
   }
   __syncthreads();                                    // the barriers are set up
   float gval = 0.f;
-  if (gptr) gval = __ldg(gptr + (int64_t)eps_row(first) * p.pitch);
+  if (gptr) gval = __ldcg(gptr + (int64_t)eps_row(first) * p.pitch);
   auto wait_row = [&](int r) {                        // after a failure nothing is waited for
     if (ok) ok = mbar_wait(&s.full[slot(r)], parity(r));
   };
@@ -165,7 +168,7 @@ __global__ void __launch_bounds__(WARPS * 32, 5)
       float v;
       if (gptr) {
         v = gf < 3 && !p.pery && (r < 0 || r >= p.ny) ? 0.f : gval;
-        if (r < last) gval = __ldg(gptr + (int64_t)eps_row(r + 1) * p.pitch);
+        if (r < last) gval = __ldcg(gptr + (int64_t)eps_row(r + 1) * p.pitch);
       } else {
         v = R[3][gsrc - xs];
       }
@@ -337,6 +340,8 @@ __device__ __forceinline__ void post_side(const PostSmem<T> &s, int sx, int sy, 
 template <typename T>
 __global__ void __launch_bounds__(GX * GY) adjoint_post_tau0_kernel(const __grid_constant__ PostArgs<T> p) {
   __shared__ PostSmem<T> s;
+  grid_wait();
+  grid_trigger();
   const int tid = threadIdx.x, tx = tid % GX, ty = tid / GX;
   const int x0 = p.bx0 + blockIdx.x * GX, y0 = p.by0 + blockIdx.y * GY;
   const int gx = x0 + tx, gy = y0 + ty;
@@ -422,8 +427,7 @@ cudaError_t post_t(const CartGeom &g, const AdjointArgs &a, const int b[4], cuda
   p.X = make_axis<T>(a.C, a.c, g.h[0], g.h[1], 1.0);
   p.Y = make_axis<T>(a.C, a.c, g.h[1], g.h[0], -1.0);
   const dim3 grid((b[1] - b[0] + GX - 1) / GX, (b[3] - b[2] + GY - 1) / GY);
-  adjoint_post_tau0_kernel<T><<<grid, GX * GY, 0, st>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(adjoint_post_tau0_kernel<T>, grid, GX * GY, 0, st, p);
 }
 
 Axis make_adj_axis(const double C[5], double c, double hn, double ht, double sign) {
@@ -489,8 +493,7 @@ cudaError_t launch_adjoint_tau0(const CartGeom &g, const AdjointArgs &a, cudaStr
   if (!encode_f32_map(&tmL, p.lam, 3, dim, stride, box) ||
       !encode_f32_map(&tmE, p.eps, 2, dim, stride, box))
     return cudaErrorInvalidValue;
-  adjoint_tau0_kernel<<<(unsigned)grid, nw * 32, smem, st>>>(tmL, tmE, p);
-  return cudaGetLastError();
+  return launch_pdl(adjoint_tau0_kernel, (unsigned)grid, nw * 32, smem, st, tmL, tmE, p);
 }
 
 }  // namespace gks

@@ -18,6 +18,7 @@
 
 #include "gks_flux2.cuh"
 #include "gks_internal.h"
+#include "gks_pdl.cuh"
 #include "gks_rcp.cuh"
 #include "gks_tau0_2d.cuh"
 
@@ -28,6 +29,8 @@ template <typename T>
 constexpr int NT = sizeof(T) == 4 ? 512 : 256;   // threads per CTA
 constexpr int kMaxSteps = kSmallSteps;
 constexpr int NF = 22;                // values a cell of the region keeps in shared memory
+constexpr int PW = 32;                // the region's side at most: constant strides in shared memory
+constexpr int N = PW * PW;
 
 template <typename T>
 struct SmallArgs {
@@ -70,7 +73,9 @@ __device__ __forceinline__ int image(int i, int n, int periodic, int pec_lo, int
 template <typename T, bool LIMIT>
 __global__ void __launch_bounds__(NT<T>) cart2d_small_kernel(const __grid_constant__ SmallArgs<T> p) {
   extern __shared__ __align__(16) unsigned char raw[];
-  const int S = p.steps, RW = p.tw + 4 * S, RH = p.th + 4 * S, N = RW * RH;
+  grid_wait();
+  grid_trigger();
+  const int S = p.steps, RW = p.tw + 4 * S, RH = p.th + 4 * S;
   T *sm = reinterpret_cast<T *>(raw);
   T *fe = sm, *fa = sm + N, *fb = sm + 2 * N;         // Ez, Hx, Hy
   T *ep = sm + 3 * N, *rx = sm + 4 * N, *ry = sm + 5 * N, *ri = sm + 6 * N;   // eps; 1/(eps sums), 1/eps
@@ -94,7 +99,7 @@ __global__ void __launch_bounds__(NT<T>) cart2d_small_kernel(const __grid_consta
     const unsigned M = ((1u << 20) + w - 1) / w;      // i / w as a product: exact for i w < 2^20
     for (unsigned i = tid; i < n; i += NT<T>) {
       const int r = (int)((i * M) >> 20), q = (int)(i - r * w);
-      body((m + r) * RW + m + q, X0 + m + q, Y0 + m + r);
+      body((m + r) * PW + m + q, X0 + m + q, Y0 + m + r);
     }
   };
   each(0, 0, [&](int i, int x, int y) {
@@ -109,7 +114,7 @@ __global__ void __launch_bounds__(NT<T>) cart2d_small_kernel(const __grid_consta
   __syncthreads();
   each(1, 0, [&](int i, int, int) {
     rx[i] = rcp_normal(ep[i - 1] + ep[i]);
-    ry[i] = rcp_normal(ep[i - RW] + ep[i]);
+    ry[i] = rcp_normal(ep[i - PW] + ep[i]);
     ri[i] = rcp_normal(ep[i]);
   });
   const bool wall = outside(X0, Y0) || outside(X0 + RW - 1, Y0 + RH - 1);   // uniform over the CTA
@@ -122,7 +127,7 @@ __global__ void __launch_bounds__(NT<T>) cart2d_small_kernel(const __grid_consta
         bool xm = false, ym = false;
         const int cx = p.perx ? x : image(x, p.nx, 0, p.pec[0], p.pec[1], xm);
         const int cy = p.pery ? y : image(y, p.ny, 0, p.pec[2], p.pec[3], ym);
-        const int j = (cy - Y0) * RW + cx - X0;
+        const int j = (cy - Y0) * PW + cx - X0;
         if (cx < X0 || cx >= X0 + RW || cy < Y0 || cy >= Y0 + RH) return;
         const T e = fe[j], a = fa[j], b = fb[j];
         fe[i] = xm != ym ? -e : e;
@@ -133,8 +138,8 @@ __global__ void __launch_bounds__(NT<T>) cart2d_small_kernel(const __grid_consta
     }
     each(2 * s + 1, 0, [&](int i, int x, int y) {
       const T e = fe[i], a = fa[i], b = fb[i], k = ep[i];
-      const T ex = raw_slope<LIMIT>(fe[i - 1], e, fe[i + 1]), ey = raw_slope<LIMIT>(fe[i - RW], e, fe[i + RW]);
-      const T bx = raw_slope<LIMIT>(fb[i - 1], b, fb[i + 1]), ay = raw_slope<LIMIT>(fa[i - RW], a, fa[i + RW]);
+      const T ex = raw_slope<LIMIT>(fe[i - 1], e, fe[i + 1]), ey = raw_slope<LIMIT>(fe[i - PW], e, fe[i + PW]);
+      const T bx = raw_slope<LIMIT>(fb[i - 1], b, fb[i + 1]), ay = raw_slope<LIMIT>(fa[i - PW], a, fa[i + PW]);
       const T ue = k * e, ux = k * ex, uy = k * ey;
       const bool gxz = (nxl && x < 0) || (nxh && x >= p.nx), gyz = (nyl && y < 0) || (nyh && y >= p.ny);
       auto sides = [&](const AxisK<T> &K, T bb, T en, T bn, T un, T at, bool zero, T *lo, T *hi) {
@@ -154,7 +159,7 @@ __global__ void __launch_bounds__(NT<T>) cart2d_small_kernel(const __grid_consta
     // faces left of and below a cell; GH of y goes over ly's P, which only this thread reads
     each(2 * s + 2, -1, [&](int i, int, int) {
       const T a = rx[i], b = ry[i];
-      const int j = i - 1, k = i - RW;
+      const int j = i - 1, k = i - PW;
       const T gex = mad(p.X.kE * a, hx[j + N] + lx[i + N], hx[j] + lx[i]);
       const T ghx = a * (hx[j + 2 * N] + lx[i + 2 * N]);
       const T gey = mad(p.Y.kE * b, hy[k + N] + ly[i + N], hy[k] + ly[i]);
@@ -167,7 +172,7 @@ __global__ void __launch_bounds__(NT<T>) cart2d_small_kernel(const __grid_consta
     __syncthreads();
     each(2 * s + 2, 0, [&](int i, int x, int y) {
       if (outside(x, y)) return;
-      T dE = mad(p.X.sE, gx[i] - gx[i + 1], p.Y.sE * (gy[i] - gy[i + RW]));
+      T dE = mad(p.X.sE, gx[i] - gx[i + 1], p.Y.sE * (gy[i] - gy[i + PW]));
       if (p.src) {
         bool m;
         const int cx = image(x, p.nx, p.perx, 0, 0, m), cy = image(y, p.ny, p.pery, 0, 0, m);
@@ -175,7 +180,7 @@ __global__ void __launch_bounds__(NT<T>) cart2d_small_kernel(const __grid_consta
           dE -= p.amp[s] * p.src[(int64_t)cy * p.pitch + cx];
       }
       fe[i] = mad(dE, ri[i], fe[i]);
-      fa[i] = mad(p.Y.sH, ly[i] - ly[i + RW], fa[i]);
+      fa[i] = mad(p.Y.sH, ly[i] - ly[i + PW], fa[i]);
       fb[i] = mad(p.X.sH, gx[i + N] - gx[i + 1 + N], fb[i]);
     });
     __syncthreads();
@@ -206,7 +211,7 @@ int sm_count() {
 // Tile and steps per launch with the least estimated time per step: a launch with its loads, the
 // phases' latency per step, and the work of the shrinking region on one SM.
 SmallPlan plan(const CartGeom &g, bool fp64, int most) {
-  const double launch = 3.0, phase = fp64 ? 1.2 : 0.8, cell = fp64 ? 0.0200 : 0.0016;   // us
+  const double launch = 2.2, phase = fp64 ? 1.2 : 1.0, cell = fp64 ? 0.0120 : 0.0020;   // us
   const int sms = sm_count();
   SmallPlan best;
   static const int sizes[] = {4, 6, 8, 10, 12, 16, 20, 24};
@@ -217,7 +222,7 @@ SmallPlan plan(const CartGeom &g, bool fp64, int most) {
       if (ctas > sms) continue;
       double work = 0.0;
       for (int S = 1; S <= std::min(most, kMaxSteps); ++S) {
-        if ((int64_t)(tw + 4 * S) * (th + 4 * S) * NF * (fp64 ? 8 : 4) > 200 * 1024) break;
+        if (tw + 4 * S > PW || th + 4 * S > PW) break;
         work += (double)(tw + 4 * S - 2) * (th + 4 * S - 2) * cell;
         const double us = (launch + S * phase + work) / S;
         if (us < best.us) {
@@ -249,27 +254,23 @@ cudaError_t launch_t(const CartGeom &g, const CartStepArgs &a, const SmallPlan &
   p.tw = pl.tw; p.th = pl.th; p.steps = pl.steps;
   p.tiles_x = (g.nx + pl.tw - 1) / pl.tw;
   const int grid = p.tiles_x * ((g.ny + pl.th - 1) / pl.th);
-  const int smem = (pl.tw + 4 * pl.steps) * (pl.th + 4 * pl.steps) * NF * (int)sizeof(T);
+  constexpr int smem = N * NF * (int)sizeof(T);
   auto kern = a.limiter ? cart2d_small_kernel<T, true> : cart2d_small_kernel<T, false>;
   static bool attr = false;
   if (!attr) {
     cudaFuncSetAttribute(cart2d_small_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         200 * 1024);
+                         smem);
     cudaFuncSetAttribute(cart2d_small_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         200 * 1024);
+                         smem);
     attr = true;
   }
-  kern<<<grid, NT<T>, smem, st>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(kern, grid, NT<T>, smem, st, p);
 }
 
 }  // namespace
 
-SmallPlan cart2d_small_plan(const CartGeom &g, const CartStepArgs &a, bool fp64, int64_t most) {
-  if (!cart2d_tau0_supported(g, a, fp64) || a.window[0] != 0 || a.window[1] != g.nx ||
-      a.window[2] != 0 || a.window[3] != g.ny || most < 1)
-    return SmallPlan();
-  SmallPlan pl = plan(g, fp64, (int)std::min<int64_t>(most, kMaxSteps));
+SmallPlan cart2d_small_plan(const CartGeom &g, bool fp64, int most) {
+  SmallPlan pl = plan(g, fp64, most);
   const double march = fp64 ? 12.0 : 6.0;             // the marching kernels' step on such a grid
   if (!(pl.us < march)) pl.steps = 0;
   return pl;

@@ -28,6 +28,7 @@
 
 #include "gks_flux2.cuh"
 #include "gks_internal.h"
+#include "gks_pdl.cuh"
 #include "gks_rcp.cuh"
 #include "gks_tau0_2d.cuh"
 #include "gks_tma.cuh"
@@ -124,12 +125,13 @@ __device__ __forceinline__ void face(const Side<V> &l, const Side<V> &r, const V
 }
 
 // Arguments shared by both kernels.
+// (not __restrict__: an early-started kernel must not use the read-only path, gks_pdl.cuh)
 template <typename T>
 struct Args {
-  const T *__restrict__ V;
-  T *__restrict__ Vout;
-  const T *__restrict__ eps;
-  const T *__restrict__ src;
+  const T *V;
+  T *Vout;
+  const T *eps;
+  const T *src;
   int sx0, sx1, sy0, sy1;
   T src_amp;
   int nx, ny;
@@ -200,6 +202,8 @@ __global__ void __launch_bounds__(WARPS * 32, 6)
                        const __grid_constant__ CUtensorMap tmE,
                        const __grid_constant__ Args<float> p) {
   extern __shared__ __align__(128) unsigned char smem_s[];
+  grid_wait();
+  grid_trigger();
   Stage &s = *reinterpret_cast<Stage *>(smem_s);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int tile = blockIdx.x % p.ntiles, chunk = blockIdx.x / p.ntiles;
@@ -268,7 +272,7 @@ __global__ void __launch_bounds__(WARPS * 32, 6)
   }
   __syncthreads();                                    // the barriers are set up
   float gval = 0.f;
-  if (EDGE && gptr) gval = __ldg(gptr + (int64_t)grid_row(first) * p.pitch);
+  if (EDGE && gptr) gval = __ldcg(gptr + (int64_t)grid_row(first) * p.pitch);
 
   auto wait_row = [&](int r) {                        // after a failure nothing is waited for
     if (ok) ok = mbar_wait(&s.full[slot(r)], parity(r));
@@ -282,7 +286,7 @@ __global__ void __launch_bounds__(WARPS * 32, 6)
       float v;
       if (EDGE && gptr) {
         v = gval;
-        if (r < last) gval = __ldg(gptr + (int64_t)grid_row(r + 1) * p.pitch);
+        if (r < last) gval = __ldcg(gptr + (int64_t)grid_row(r + 1) * p.pitch);
       } else {
         v = gsign * R[gf][gsrc - xs];
       }
@@ -456,6 +460,8 @@ template <int NC, bool LIMIT>
 __global__ void __launch_bounds__(WARPS * 32, 2)
     cart2d_tau0_f64_kernel(const __grid_constant__ Args<double> p) {
   constexpr int WD = 32 * NC - 2;
+  grid_wait();
+  grid_trigger();
   const int lane = threadIdx.x & 31;
   const int wid = blockIdx.x * WARPS + (threadIdx.x >> 5);
   const int strip = wid % p.ntiles, chunk = wid / p.ntiles;
@@ -485,15 +491,15 @@ __global__ void __launch_bounds__(WARPS * 32, 2)
     const double *q = p.V + ro, *qe = p.eps + ro;
 #pragma unroll
     for (int i = 0; i < NC; ++i) {
-      o.e.v[i] = flip(__ldg(q + ci[i]), xm[i] != ym);
-      o.a.v[i] = flip(__ldg(q + p.cstride + ci[i]), xm[i]);
-      o.b.v[i] = flip(__ldg(q + 2 * p.cstride + ci[i]), ym);
-      o.ep.v[i] = __ldg(qe + ci[i]);
+      o.e.v[i] = flip(__ldcg(q + ci[i]), xm[i] != ym);
+      o.a.v[i] = flip(__ldcg(q + p.cstride + ci[i]), xm[i]);
+      o.b.v[i] = flip(__ldcg(q + 2 * p.cstride + ci[i]), ym);
+      o.ep.v[i] = __ldcg(qe + ci[i]);
     }
     o.ee = o.be = 0.0;
     if (rim) {
-      o.ee = flip(__ldg(q + ce), em_ != ym);
-      o.be = flip(__ldg(q + 2 * p.cstride + ce), ym);
+      o.ee = flip(__ldcg(q + ce), em_ != ym);
+      o.be = flip(__ldcg(q + 2 * p.cstride + ce), ym);
     }
     return o;
   };
@@ -680,8 +686,7 @@ cudaError_t launch_f32(const CartGeom &g, const CartStepArgs &a, cudaStream_t st
       !encode_f32_map(&tmE, p.eps, 2, dim, stride, box))
     return cudaErrorInvalidValue;
   const bool edge = p.perx || p.pery || p.pec[0] || p.pec[1] || p.pec[2] || p.pec[3];
-  kern[edge ? 1 : 0][a.limiter ? 1 : 0]<<<(unsigned)grid, nw * 32, smem, st>>>(tmV, tmE, p);
-  return cudaGetLastError();
+  return launch_pdl(kern[edge ? 1 : 0][a.limiter ? 1 : 0], (unsigned)grid, nw * 32, smem, st, tmV, tmE, p);
 }
 
 cudaError_t launch_f64(const CartGeom &g, const CartStepArgs &a, cudaStream_t st) {
@@ -714,8 +719,7 @@ cudaError_t launch_f64(const CartGeom &g, const CartStepArgs &a, cudaStream_t st
   using K = void (*)(const Args<double>);
   static const K kern[2][2] = {{cart2d_tau0_f64_kernel<1, false>, cart2d_tau0_f64_kernel<1, true>},
                                {cart2d_tau0_f64_kernel<2, false>, cart2d_tau0_f64_kernel<2, true>}};
-  kern[cols - 1][a.limiter ? 1 : 0]<<<grid, WARPS * 32, 0, st>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(kern[cols - 1][a.limiter ? 1 : 0], grid, WARPS * 32, 0, st, p);
 }
 
 }  // namespace

@@ -12,6 +12,7 @@
 #include <cuda_runtime.h>
 
 #include "gks_internal.h"
+#include "gks_pdl.cuh"
 #include "gks_pair3.cuh"
 #include "gks_rcp.cuh"
 #include "gks_tma.cuh"
@@ -57,10 +58,10 @@ struct OpS {
 };
 
 struct Args {
-  const float *__restrict__ V;
-  float *__restrict__ Vout;
-  const float *__restrict__ eps;
-  const float *__restrict__ src;
+  const float *V;                      // (not __restrict__: gks_pdl.cuh)
+  float *Vout;
+  const float *eps;
+  const float *src;
   int sx0, sx1, sy0, sy1, sz0, sz1;
   float src_amp;
   int nx, ny, nz;
@@ -167,7 +168,7 @@ __device__ __forceinline__ void fix_plane(Smem &s, const Args &a, int slot, int 
       v[u] = 0.f;
       if (i < n) {
         const int dd = s.fixd[i], arr = dd / (NR * TW);
-        v[u] = __ldg((arr < 6 ? a.V + arr * a.cstride : a.eps) + (int64_t)gz * a.plane + s.fixg[i]);
+        v[u] = __ldcg((arr < 6 ? a.V + arr * a.cstride : a.eps) + (int64_t)gz * a.plane + s.fixg[i]);
         d[u] = dd;
       }
     }
@@ -268,6 +269,8 @@ __global__ void __launch_bounds__(NTH, CTAS)
     cart3d_tau0_kernel(const __grid_constant__ CUtensorMap tmV,
                        const __grid_constant__ CUtensorMap tmE, const __grid_constant__ Args a) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
+  grid_wait();
+  grid_trigger();
   Smem &s = *reinterpret_cast<Smem *>(smem_raw);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int X0 = blockIdx.x * TCOLS, y0 = blockIdx.y * NWO;
@@ -327,7 +330,7 @@ __global__ void __launch_bounds__(NTH, CTAS)
 #pragma unroll
     for (int m = 0; m < NA; ++m) {
       const float *base = (m < 6 ? a.V + m * a.cstride : a.eps) + o;
-      Wm[m] = pk(__ldg(base + c0), __ldg(base + c1));
+      Wm[m] = pk(__ldcg(base + c0), __ldcg(base + c1));
     }
   }
   {
@@ -629,8 +632,7 @@ cudaError_t launch_cart3d_tau0(const CartGeom &g, const CartStepArgs &a, cudaStr
   CUtensorMap tmV, tmE;
   if (!encode_map(&tmV, p.V, g, 4) || !encode_map(&tmE, p.eps, g, 3)) return cudaErrorInvalidValue;
   dim3 grid(gx, gy, zchunks);
-  cart3d_tau0_kernel<<<grid, NTH, smem, st>>>(tmV, tmE, p);
-  return cudaGetLastError();
+  return launch_pdl(cart3d_tau0_kernel, grid, NTH, smem, st, tmV, tmE, p);
 }
 
 }  // namespace gks

@@ -13,6 +13,7 @@
 
 #include "gks_flux3.cuh"
 #include "gks_internal.h"
+#include "gks_pdl.cuh"
 
 namespace gks {
 namespace {
@@ -52,9 +53,10 @@ __device__ __forceinline__ void load_cell_w(const double *p, double w[kTetCellW]
 }
 
 template <typename T>
-__global__ void tet_gradient_kernel(const T *__restrict__ V, const int32_t *__restrict__ cnb,
-                                    const T *__restrict__ cw, int64_t nt, int pec,
-                                    T *__restrict__ G) {
+__global__ void tet_gradient_kernel(const T *V, const int32_t *__restrict__ cnb,
+                                    const T *__restrict__ cw, int64_t nt, int pec, T *G) {
+  grid_wait();
+  grid_trigger();
   const int64_t i = blockIdx.x * (int64_t)TBT<T> + threadIdx.x;
   if (i >= nt) return;
   // every load is issued before the arithmetic: the four neighbour indices in one vector load,
@@ -231,7 +233,7 @@ struct TetK0 {
 // A side's share of the tau = 0 face flux (see tet_face_tau0_kernel), added into PE, QE, QH; m = n/c
 // for the low side, -n/c for the high side.  The gradient rows are loaded a field at a time.
 template <typename T>
-__device__ __forceinline__ void tet_side_tau0(const T *__restrict__ V, const T *__restrict__ G, T eps,
+__device__ __forceinline__ void tet_side_tau0(const T *V, const T *G, T eps,
                                               int64_t nt, int64_t cell, const T d[3], const T m[3],
                                               const TetK0<T> &K, T PE[3], T QE[3], T QH[3]) {
   const T m1[3] = {K.h1 * m[0], K.h1 * m[1], K.h1 * m[2]};
@@ -268,10 +270,11 @@ __device__ __forceinline__ void tet_side_tau0(const T *__restrict__ V, const T *
 // (tangentially) and cancels QH.
 template <typename T>
 __global__ void __launch_bounds__(TBT<T>, sizeof(T) == 4 ? 4 : 1)
-    tet_face_tau0_kernel(const T *__restrict__ V, const T *__restrict__ G,
-                         const T *__restrict__ eps, const int32_t *__restrict__ fL,
+    tet_face_tau0_kernel(const T *V, const T *G, const T *eps, const int32_t *__restrict__ fL,
                          const int32_t *__restrict__ fR, const T *__restrict__ fgeo, int64_t nt,
-                         int64_t nf, int pec, const TetK0<T> K, T *__restrict__ F) {
+                         int64_t nf, int pec, const TetK0<T> K, T *F) {
+  grid_wait();
+  grid_trigger();
   const int64_t f = blockIdx.x * (int64_t)TBT<T> + threadIdx.x;
   if (f >= nf) return;
   const int32_t L = fL[f], R = fR[f];
@@ -323,13 +326,12 @@ __device__ __forceinline__ void load_cell_u(const double *p, double w[4]) {
 }
 
 template <typename T>
-__global__ void tet_update_kernel(const T *__restrict__ V, T *__restrict__ Vout,
-                                  const T *__restrict__ eps, const T *__restrict__ mu,
-                                  const T *__restrict__ src, T src_amp,
-                                  const int32_t *__restrict__ cface,
-                                  const T *__restrict__ cu, const T *__restrict__ F, int64_t nt,
-                                  int64_t nf,
-                                  int *__restrict__ flag) {
+__global__ void tet_update_kernel(const T *V, T *Vout, const T *eps, const T *mu, const T *src,
+                                  T src_amp, const int32_t *__restrict__ cface,
+                                  const T *__restrict__ cu, const T *F, int64_t nt, int64_t nf,
+                                  int *flag) {
+  grid_wait();
+  grid_trigger();
   const int64_t i = blockIdx.x * (int64_t)TBT<T> + threadIdx.x;
   bool bad = false;
   if (i < nt) {
@@ -337,7 +339,9 @@ __global__ void tet_update_kernel(const T *__restrict__ V, T *__restrict__ Vout,
     load_cell_u(cu + kTetCellU * i, w);
     const int4 fc = __ldg(reinterpret_cast<const int4 *>(cface) + i);
     const int32_t fk[4] = {fc.x, fc.y, fc.z, fc.w};
-    T d[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
+    T d[6] = {T(0), T(0), T(0), T(0), T(0), T(0)}, v[6];
+#pragma unroll
+    for (int c = 0; c < 6; ++c) v[c] = V[c * nt + i];
 #pragma unroll
     for (int k = 0; k < 4; ++k)
 #pragma unroll
@@ -348,7 +352,7 @@ __global__ void tet_update_kernel(const T *__restrict__ V, T *__restrict__ Vout,
     T sum = T(0);
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
-      const T nv = V[c * nt + i] + d[c] * (c < 3 ? ie : im);
+      const T nv = v[c] + d[c] * (c < 3 ? ie : im);
       Vout[c * nt + i] = nv;
       sum += nv;
     }
@@ -428,29 +432,29 @@ cudaError_t step_t(const TetDev &g, const void *Vin, void *Vout, const void *eps
   T *F = static_cast<T *>(g.Fscratch);
   const T *fgeo = static_cast<const T *>(g.fgeo);
   const T *cw = static_cast<const T *>(g.cw), *cu = static_cast<const T *>(g.cu);
-  tet_gradient_kernel<T><<<blocks_for<T>(g.nt), TBT<T>, 0, st>>>(V, g.cnb, cw, g.nt, g.pec, G);
-  if (!mu && C[1] == 0.0 && C[3] == 0.0 && C[4] == 0.0) {
-    const TetK0<T> K0 = {T(0.5 * C[0]), T(0.5 * C[2]), T(1.0 / c)};
-    tet_face_tau0_kernel<T><<<blocks_for<T>(g.nf), TBT<T>, 0, st>>>(
-        V, G, static_cast<const T *>(eps), g.fL, g.fR, fgeo, g.nt, g.nf, g.pec, K0, F);
-    tet_update_kernel<T><<<blocks_for<T>(g.nt), TBT<T>, 0, st>>>(
-        V, static_cast<T *>(Vout), static_cast<const T *>(eps), nullptr,
-        static_cast<const T *>(src), T(src_amp), g.cface, cu, F, g.nt, g.nf, flag);
-    return cudaGetLastError();
-  }
+  const T *ep = static_cast<const T *>(eps), *m = static_cast<const T *>(mu);
+  const unsigned ct = blocks_for<T>(g.nt), cf = blocks_for<T>(g.nf);
+  // geometry comes through the read-only path (set up once); what a step writes does not (gks_pdl.cuh)
+  cudaError_t e = launch_pdl(tet_gradient_kernel<T>, ct, TBT<T>, 0, st, V, g.cnb, cw, g.nt, g.pec, G);
+  if (e != cudaSuccess) return e;
   const K3<T> K = make_k3<T>(C, 1.0, c);     // fluxes carry dt (C_i), areas applied per face
   const F3K<T> FK = make_f3k<T>(C, 1.0, c);
-  if (mu)
-    tet_face_kernel<T, true><<<blocks_for<T>(g.nf), TBT<T>, 0, st>>>(
-        V, G, static_cast<const T *>(eps), static_cast<const T *>(mu), g.fL, g.fR, fgeo, g.nt,
-        g.nf, g.pec, K, FK, F);
-  else
-    tet_face_kernel<T, false><<<blocks_for<T>(g.nf), TBT<T>, 0, st>>>(
-        V, G, static_cast<const T *>(eps), nullptr, g.fL, g.fR, fgeo, g.nt, g.nf, g.pec, K, FK, F);
-  tet_update_kernel<T><<<blocks_for<T>(g.nt), TBT<T>, 0, st>>>(
-      V, static_cast<T *>(Vout), static_cast<const T *>(eps), static_cast<const T *>(mu),
-      static_cast<const T *>(src), T(src_amp), g.cface, cu, F, g.nt, g.nf, flag);
-  return cudaGetLastError();
+  if (!mu && C[1] == 0.0 && C[3] == 0.0 && C[4] == 0.0) {
+    const TetK0<T> K0 = {T(0.5 * C[0]), T(0.5 * C[2]), T(1.0 / c)};
+    e = launch_pdl(tet_face_tau0_kernel<T>, cf, TBT<T>, 0, st, V, G, ep, g.fL, g.fR, fgeo, g.nt, g.nf,
+                   g.pec, K0, F);
+  } else {
+    if (mu)
+      tet_face_kernel<T, true><<<cf, TBT<T>, 0, st>>>(V, G, ep, m, g.fL, g.fR, fgeo, g.nt, g.nf, g.pec,
+                                                      K, FK, F);
+    else
+      tet_face_kernel<T, false><<<cf, TBT<T>, 0, st>>>(V, G, ep, nullptr, g.fL, g.fR, fgeo, g.nt, g.nf,
+                                                       g.pec, K, FK, F);
+    e = cudaGetLastError();
+  }
+  if (e != cudaSuccess) return e;
+  return launch_pdl(tet_update_kernel<T>, ct, TBT<T>, 0, st, V, static_cast<T *>(Vout), ep, m,
+                    static_cast<const T *>(src), T(src_amp), g.cface, cu, F, g.nt, g.nf, flag);
 }
 
 int grid_capped(int64_t n) {
