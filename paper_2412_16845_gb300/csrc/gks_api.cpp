@@ -433,16 +433,19 @@ gks_status gks_set_materials(gks_ctx *ctx, const double *eps, const double *mu) 
   if (!eps) return fail(ctx, GKS_E_ARG, "eps is NULL");
   if (mu && ctx->phm) return fail(ctx, GKS_E_UNSUPPORTED, "divergence cleaning needs mu = 1");
   // lattice speed: the fastest wave, light 1/sqrt(eps mu) or a cleaning wave (mu = 1)
-  double cmax = cleaning_speed(ctx);
-  bool normal = true;
+  // (1/sqrt is monotone, rounding included: the fastest light is that of the least eps mu)
+  double least = HUGE_VAL, elo = HUGE_VAL, ehi = 0.0;
   for (int64_t i = 0; i < ctx->ncell; ++i) {
     const double e = eps[i], m = mu ? mu[i] : 1.0;
     if (!finite_positive(e) || !finite_positive(m))
       return fail(ctx, GKS_E_ARG, "eps and mu must be finite and > 0 (cell " +
                                       std::to_string(i) + ")");
-    cmax = std::fmax(cmax, 1.0 / std::sqrt(e * m));
-    normal = normal && normal_eps(e);
+    least = std::min(least, e * m);
+    elo = std::min(elo, e);
+    ehi = std::max(ehi, e);
   }
+  const double cmax = std::fmax(cleaning_speed(ctx), 1.0 / std::sqrt(least));
+  const bool normal = normal_eps(elo) && normal_eps(ehi);
   gks_status s;
   if ((s = upload_cells(ctx, eps, 1, ctx->eps)) != GKS_OK) return s;
   if (mu) {
@@ -617,23 +620,44 @@ gks::CartStepArgs step_args(const gks_ctx *ctx, const int win[4]) {
 gks_status step_impl(gks_ctx *ctx, int64_t n_steps, const int win[4], bool objective) {
   gks::CartStepArgs a = step_args(ctx, win);
   // windowed steps (objective = false) march: their windows are recomputed step by step
-  const bool small = objective && ctx->kind == GKS_CARTESIAN && ctx->dim == 2 && !ctx->phm;
+  const bool small2 = objective && ctx->kind == GKS_CARTESIAN && ctx->dim == 2 && !ctx->phm &&
+                      gks::cart2d_tau0_supported(ctx->g, a, ctx->fp64);
+  const bool small3 = ctx->kind == GKS_CARTESIAN && ctx->dim == 3 && !ctx->phm &&
+                      gks::cart3d_tau0_f64_supported(a);
   const bool probe = objective && ctx->np > 0;       // needs the state after every step
+  auto plan2 = [ctx, probe](int64_t left) {
+    const int most = probe ? 1 : (int)std::min<int64_t>(left, gks::kSmallSteps);
+    if (!ctx->have2[most]) {
+      ctx->plan2[most] = gks::cart2d_small_plan(ctx->g, ctx->fp64, most);
+      ctx->have2[most] = true;
+    }
+    return ctx->plan2[most];
+  };
   gks::SmallPlan pl;
-  if (small) pl = gks::cart2d_small_plan(ctx->g, a, ctx->fp64, probe ? 1 : n_steps);
+  gks::SmallPlan3 pl3;
+  if (small2 && n_steps > 0) pl = plan2(n_steps);
+  if (small3) {
+    if (!ctx->have3) {
+      ctx->plan3 = gks::cart3d_small_plan(ctx->g, ctx->fp64);
+      ctx->have3 = true;
+    }
+    pl3 = ctx->plan3;
+  }
   for (int64_t n = 0; n < n_steps;) {
     a.src_amp = source_amplitude(ctx, ctx->step);
     a.V = ctx->V[ctx->cur];
     a.Vout = ctx->V[ctx->cur ^ 1];
     cudaError_t e;
     int done = 1;
-    if (pl.steps > n_steps - n)                       // the last launch takes fewer steps
-      pl = gks::cart2d_small_plan(ctx->g, a, ctx->fp64, n_steps - n);
+    if (pl.steps > n_steps - n) pl = plan2(n_steps - n);   // the last launch takes fewer steps
     if (pl.steps > 0) {
       double amp[gks::kSmallSteps];
       done = pl.steps;
       for (int s = 0; s < done; ++s) amp[s] = source_amplitude(ctx, ctx->step + s);
       e = gks::launch_cart2d_small(ctx->g, a, pl, amp, ctx->fp64, ctx->st);
+      ctx->launches += 1;
+    } else if (pl3.tile >= 0) {
+      e = gks::launch_cart3d_small(ctx->g, a, pl3, ctx->fp64, ctx->st);
       ctx->launches += 1;
     } else if (ctx->kind == GKS_TET) {
       e = gks::launch_tet_step(ctx->tet, a.V, a.Vout, a.eps, a.mu, a.src, a.src_amp, a.C, a.c,

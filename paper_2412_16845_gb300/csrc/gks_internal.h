@@ -153,16 +153,25 @@ cudaError_t launch_cart3d_step(const CartGeom &g, const CartStepArgs &a, bool fp
 bool cart3d_side_supported(const CartGeom &g, const CartStepArgs &a, bool fp64);
 cudaError_t launch_cart3d_side(const CartGeom &g, const CartStepArgs &a, cudaStream_t st);
 // Several 2-D steps in one launch on grids too small to fill the GPU (gks_cart2d_small.cu): the tile
-// and steps per launch (0: the marching kernels are better), at most `most` steps; and the launch,
-// with the source amplitude of each step.
+// and steps per launch (0: the marching kernels are better), at most `most` steps, for a step that
+// cart2d_tau0_supported(); and the launch, with the source amplitude of each step.
 constexpr int kSmallSteps = 8;
 struct SmallPlan {
   int tw = 0, th = 0, steps = 0;
   double us = 1e300;                  // estimated time per step
 };
-SmallPlan cart2d_small_plan(const CartGeom &g, const CartStepArgs &a, bool fp64, int64_t most);
+SmallPlan cart2d_small_plan(const CartGeom &g, bool fp64, int most);
 cudaError_t launch_cart2d_small(const CartGeom &g, const CartStepArgs &a, const SmallPlan &pl,
                                 const double *amp, bool fp64, cudaStream_t st);
+// One step of a small 3-D grid (gks_cart3d_small.cu): the tile (-1: march), for a step that
+// cart3d_tau0_f64_supported() (the conditions on the flux are the same); and the launch.
+struct SmallPlan3 {
+  int tile = -1;
+  double us = 1e300;                  // estimated time per step
+};
+SmallPlan3 cart3d_small_plan(const CartGeom &g, bool fp64);
+cudaError_t launch_cart3d_small(const CartGeom &g, const CartStepArgs &a, const SmallPlan3 &pl,
+                                bool fp64, cudaStream_t st);
 // FP32 3-D step with tau = 0 where the side-split kernel would run (gks_cart3d_tau0.cu).
 bool cart3d_tau0_supported(const CartGeom &g, const CartStepArgs &a);
 cudaError_t launch_cart3d_tau0(const CartGeom &g, const CartStepArgs &a, cudaStream_t st);
@@ -231,6 +240,10 @@ struct gks_ctx {
   double min_h = 1.0;
   bool fields_written = false;
   int64_t launches = 0;
+  // launch plans of small grids, which the grid alone decides (made at the first step that asks)
+  gks::SmallPlan plan2[gks::kSmallSteps + 1];
+  gks::SmallPlan3 plan3;
+  bool have2[gks::kSmallSteps + 1] = {}, have3 = false;
   // objective / adjoint (2-D Cartesian)
   int64_t *probe_off = nullptr;   // [np] state offsets of the probe cells
   double *probe_w = nullptr;      // [np] |Omega_i|

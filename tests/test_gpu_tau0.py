@@ -94,22 +94,24 @@ def test_2d_extreme_permittivity_keeps_its_results():
     assert rel_l2(out["fp32"], out["fp64"]) <= 2e-5
 
 
-# 3-D FP64: strips of 30 cells along any axis, up to 8 rows and any number of planes per warp
-@pytest.mark.parametrize("limiter", [None, "vanleer"])
-@pytest.mark.parametrize("n,bc", [
-    ((30, 9, 5), "nnnnnn"), ((31, 8, 3), "ppnnmm"), ((61, 3, 2), "mmppnn"), ((7, 30, 12), "nmnnpp"),
-    ((5, 6, 62), "pppppp"), ((1, 1, 1), "nnnnnn"), ((3, 17, 2), "nnppnm"), ((2, 2, 33), "mmmmmm"),
+# 3-D small grids: one tile per CTA
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("n,bc,limiter", [
+    ((45, 34, 27), "nnpppp", None), ((17, 5, 9), "mmnnpp", None), ((1, 1, 1), "pppppp", None),
+    ((30, 3, 2), "nmppmn", None), ((20, 20, 20), "nnnnnn", "vanleer"), ((2, 33, 7), "ppmmnn", "vanleer"),
 ])
-def test_3d_fp64_tiles(n, bc, limiter):
+def test_3d_small_grids(n, bc, limiter, precision):
     sides = tuple({"n": "nrbc", "p": "periodic", "m": "pec"}[b] for b in bc)
-    _check(_grid(n, sides, seed=sum(n), limiter=limiter), "fp64", 5)
+    _check(_grid(n, sides, seed=n[0] + n[1], limiter=limiter), precision, 6)
 
 
-# 3-D FP32: tiles of 64 columns x 10 rows, chunks of planes
-@pytest.mark.parametrize("n,bc", [
-    ((64, 10, 9), "nnnnnn"), ((65, 11, 3), "ppnnpp"), ((63, 21, 2), "nnppnn"), ((3, 2, 30), "nnnnnn"),
-    ((130, 9, 5), "pppppp"), ((1, 1, 1), "nnnnnn"), ((7, 12, 1), "nnnnpp"),
+# The marching kernels, on grids just past what takes one tile per CTA.  FP64: strips of 30 cells, up
+# to 8 rows and any number of planes per warp; FP32: tiles of 64 columns x 10 rows, chunks of planes.
+@pytest.mark.parametrize("n,bc,precision,limiter", [
+    ((31, 73, 72), "nnmmpp", "fp64", None), ((121, 41, 33), "ppnnnm", "fp64", "vanleer"),
+    ((59, 2, 1400), "mmnnpp", "fp64", None), ((65, 51, 50), "nnppnn", "fp32", None),
+    ((129, 41, 31), "ppnnpp", "fp32", None), ((63, 1, 2600), "nnppnn", "fp32", None),
 ])
-def test_3d_fp32_tiles(n, bc):
-    sides = tuple({"n": "nrbc", "p": "periodic"}[b] for b in bc)
-    _check(_grid(n, sides, seed=sum(n) + 1), "fp32", 7)
+def test_3d_marching_tiles(n, bc, precision, limiter):
+    sides = tuple({"n": "nrbc", "p": "periodic", "m": "pec"}[b] for b in bc)
+    _check(_grid(n, sides, seed=sum(n), limiter=limiter), precision, 2)
