@@ -611,6 +611,7 @@ cudaError_t launch_cart3d_step(const CartGeom &g, const CartStepArgs &a, bool fp
 
 cudaError_t launch_cart3d_phm_step(const CartGeom &g, const CartStepArgs &a, double chi,
                                    double gamma, bool fp64, cudaStream_t st) {
+  if (cart3d_tau0_f64_supported(a)) return launch_cart3d_phm_tau0(g, a, chi, gamma, fp64, st);
   return fp64 ? launch3_t<double, 8>(g, a, chi, gamma, st)
               : launch3_t<float, 8>(g, a, chi, gamma, st);
 }

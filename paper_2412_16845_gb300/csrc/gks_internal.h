@@ -182,6 +182,9 @@ cudaError_t launch_cart3d_tau0_f64(const CartGeom &g, const CartStepArgs &a, cud
 // Divergence-cleaning system on a 3-D grid: V = (E, H, phi, psi), 8 components.
 cudaError_t launch_cart3d_phm_step(const CartGeom &g, const CartStepArgs &a, double chi,
                                    double gamma, bool fp64, cudaStream_t st);
+// The same with tau = 0, for a step that cart3d_tau0_f64_supported() (gks_cart3d_phm_tau0.cu).
+cudaError_t launch_cart3d_phm_tau0(const CartGeom &g, const CartStepArgs &a, double chi,
+                                   double gamma, bool fp64, cudaStream_t st);
 cudaError_t launch_cart2d_psi_step(const CartGeom &g, const CartStepArgs &a, double gamma,
                                    bool fp64, cudaStream_t st);
 cudaError_t launch_user_to_cart(const CartGeom &g, int ncomp, const double *user, void *dst,

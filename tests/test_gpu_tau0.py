@@ -115,3 +115,19 @@ def test_3d_small_grids(n, bc, limiter, precision):
 def test_3d_marching_tiles(n, bc, precision, limiter):
     sides = tuple({"n": "nrbc", "p": "periodic", "m": "pec"}[b] for b in bc)
     _check(_grid(n, sides, seed=sum(n), limiter=limiter), precision, 2)
+
+
+# divergence cleaning, 3-D: tiles of 30 x 10 (FP32) or 30 x 6 (FP64) columns, chunks of planes
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("n,bc,limiter", [
+    ((30, 10, 7), "nnnnnn", None), ((31, 11, 6), "mnnmnn", None), ((29, 7, 5), "ppnnmm", None),
+    ((61, 21, 40), "nnppnn", None), ((1, 1, 1), "nnnnnn", None), ((2, 13, 1), "mmnnpp", None),
+    ((33, 6, 9), "nmppnn", "vanleer"), ((30, 31, 3), "pppppp", "vanleer"),
+])
+def test_3d_cleaning_tiles(n, bc, limiter, precision):
+    sides = tuple({"n": "nrbc", "p": "periodic", "m": "pec"}[b] for b in bc)
+    w = _grid(n, sides, seed=sum(n) + 11, limiter=limiter)
+    rng = np.random.default_rng(n[0])
+    w.fields0 = np.concatenate([w.fields0, rng.standard_normal((2, w.fields0.shape[1]))])
+    w.phm, w.cfl = (0.7, 1.3), 0.25
+    _check(w, precision, 5)
