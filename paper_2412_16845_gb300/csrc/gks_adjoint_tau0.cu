@@ -472,17 +472,19 @@ cudaError_t launch_adjoint_tau0(const CartGeom &g, const AdjointArgs &a, cudaStr
     cudaFuncSetAttribute(adjoint_tau0_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     sms = n > 0 ? n : 1;
   }
-  // chunks as in the step: waves of five CTAs per SM, 16 rows or more (a chunk computes two rows
-  // more), fewer while that fills idle SMs
+  // Rows a chunk (which computes two rows more): one wave of five CTAs per SM while that takes 40 rows or
+  // fewer, past that about four waves, 24 rows or more.  2048 x 2048: one wave (25 to 28 rows) 38 us, 24
+  // (1.02 waves) 44, 14 rows 36; 1448 x 1448: one wave (12) 18.9, 8: 21.6; 2900 x 2900: one wave (47)
+  // 61.2, 24: 61.6, 16: 62.8.
   const int wrows = p.wy1 - p.wy0, strips = (p.wx1 - p.wx0 + W - 1) / W;
   const int nw = std::min(WARPS, strips);
   p.ntiles = (strips + nw - 1) / nw;
   const int64_t resident = (int64_t)sms * 5;
-  int64_t chunks = std::max<int64_t>(1, 4 * resident / p.ntiles);
-  int rows = (int)((wrows + chunks - 1) / chunks);
-  if (rows < 24) {
-    chunks = std::max<int64_t>(1, resident / p.ntiles);
-    rows = std::min(24, std::max(4, (int)((wrows + chunks - 1) / chunks)));
+  const int64_t fit = std::max<int64_t>(1, resident / p.ntiles);
+  int rows = std::max(4, (int)((wrows + fit - 1) / fit));
+  if (rows > 40) {
+    const int64_t chunks = std::max<int64_t>(1, 4 * resident / p.ntiles);
+    rows = std::max(24, (int)((wrows + chunks - 1) / chunks));
   }
   p.rows = rows;
   const int64_t grid = (int64_t)p.ntiles * ((wrows + rows - 1) / rows);

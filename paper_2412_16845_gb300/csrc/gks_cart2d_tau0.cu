@@ -667,14 +667,17 @@ cudaError_t launch_f32(const CartGeom &g, const CartStepArgs &a, cudaStream_t st
   const int wrows = p.wy1 - p.wy0, strips = (p.wx1 - p.wx0 + W - 1) / W;
   const int nw = std::min(WARPS, strips);
   p.ntiles = (strips + nw - 1) / nw;
-  // About eight waves of six CTAs per SM on large grids (chunks of 16 rows or more: a chunk's
-  // prologue costs about a row); fewer rows, down to 2, while that fills idle SMs.
+  // Rows a chunk: one wave of six CTAs per SM while that takes 24 rows or fewer; past that about eight
+  // waves, chunks of 16 rows or more (a chunk's prologue costs about a row and a half).  At 2048 x 2048
+  // one wave of 21 or 22 rows and 8 to 14 rows take 30 to 31 us, 16 (1.3 waves) 32.4, 20 (1.02) 33.4;
+  // 1448 x 1448: one wave (10) 15.5, 8: 17.4; 2900 x 2900: 16 rows 52.2, one wave (39) 53.7;
+  // 4096 x 4096: 16 rows 90.8, 10: 93.2.
   const int64_t resident = (int64_t)sms * 6;
-  int64_t chunks = std::max<int64_t>(1, 8 * resident / p.ntiles);
-  int rows = (int)((wrows + chunks - 1) / chunks);
-  if (rows < 16) {
-    chunks = std::max<int64_t>(1, resident / p.ntiles);
-    rows = std::min(16, std::max(2, (int)((wrows + chunks - 1) / chunks)));
+  const int64_t fit = std::max<int64_t>(1, resident / p.ntiles);
+  int rows = std::max(2, (int)((wrows + fit - 1) / fit));
+  if (rows > 24) {
+    const int64_t chunks = std::max<int64_t>(1, 8 * resident / p.ntiles);
+    rows = std::max(16, (int)((wrows + chunks - 1) / chunks));
   }
   p.rows = rows;
   const int64_t grid = (int64_t)p.ntiles * ((wrows + rows - 1) / rows);
