@@ -38,8 +38,8 @@ sys.path.insert(0, ROOT)
 METRIC = "GCell-updates/s FP32 vs FP64 at stated error; % HBM roofline; adjoint/fwd cost"
 UNIT = "GCell-updates/s"
 BYTES_PER_CELL_STEP = {"fp32": 28, "fp64": 56}   # 3 fields read + written, eps read
-KERNEL_SRC = os.path.join(ROOT, "paper_2412_16845_gb300", "csrc", "gks_cart2d.cu")
-PROFILE = os.path.join(ROOT, "profiles", "cart2d_step_tm2d_cylinders_4096_fp32.md")
+KERNEL_SRC = os.path.join(ROOT, "paper_2412_16845_gb300", "csrc", "gks_cart2d_tau0.cu")
+PROFILE = os.path.join(ROOT, "profiles", "cart2d_tau0_tm2d_cylinders_4096_fp32.md")
 
 
 def _peaks():
@@ -50,8 +50,8 @@ def _peaks():
     return 6800.0, "fallback"
 
 
-KERNEL_SRC_3D = os.path.join(ROOT, "paper_2412_16845_gb300", "csrc", "gks_cart3d_side.cu")
-PROFILE_3D = os.path.join(ROOT, "profiles", "cart3d_side_step_maxwell3d_sphere_fp32.md")
+KERNEL_SRC_3D = os.path.join(ROOT, "paper_2412_16845_gb300", "csrc", "gks_cart3d_tau0.cu")
+PROFILE_3D = os.path.join(ROOT, "profiles", "cart3d_tau0_maxwell3d_sphere_fp32.md")
 
 
 def _kernel_hash(src=KERNEL_SRC):
@@ -285,11 +285,11 @@ def reduced_gpu_results(stream_ptr, path):
     np.savez(path, **out)
 
 
-# The 3-D FP32 step kernel (cart3d_side_kernel) is bound by instruction issue: its ncu summary
-# (profiles/cart3d_side_step_maxwell3d_sphere_fp32.md) counts 608 thread-instructions per cell at
-# 160^3, where 20% of the 64-column tiles lie past the grid, i.e. about 520 per cell on a grid of
+# The 3-D FP32 step kernel (cart3d_tau0_kernel) is bound by instruction issue: its ncu summary
+# (profiles/cart3d_tau0_maxwell3d_sphere_fp32.md) counts 426 thread-instructions per cell at
+# 160^3, where 20% of the 64-column tiles lie past the grid, i.e. about 355 per cell on a grid of
 # whole tiles such as 256^3.  The issue peak is 152 SMs x 4 schedulers x 32 threads x 2.07 GHz.
-INSTR_PER_CELL_3D = 520
+INSTR_PER_CELL_3D = 355
 ISSUE_PEAK_T = 152 * 4 * 32 * 2.07e9 / 1e12          # T thread-instructions/s
 
 
@@ -303,8 +303,8 @@ def roofline_3d(ncell, ms):
             "unit": "T thread-instructions/s", "frac": achieved / ISSUE_PEAK_T,
             "peak_source": "152 SMs x 4 schedulers x 32 lanes x 2.07 GHz",
             "instructions_per_cell": INSTR_PER_CELL_3D,
-            "instructions_source": "ncu, profiles/cart3d_side_step_maxwell3d_sphere_fp32.md",
-            "kernel": "cart3d_side_kernel (FP32, mu = 1)",
+            "instructions_source": "ncu, profiles/cart3d_tau0_maxwell3d_sphere_fp32.md",
+            "kernel": "cart3d_tau0_kernel (FP32, mu = 1, tau = 0)",
             "hbm": {"achieved": 52 * gcells, "peak": hbm, "unit": "GB/s",
                     "frac": 52 * gcells / hbm, "peak_source": how,
                     "traffic": _profiled_traffic(PROFILE_3D, KERNEL_SRC_3D) if ncell == 256 ** 3
@@ -477,7 +477,7 @@ def run_sharded(args, w, world, rank, local, stream):
                                       "send/recv after every step"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                          "frac": achieved / hbm, "peak_source": how, "traffic": None,
-                         "kernel": "cart2d_step_kernel_s (staged FP32, mu = 1), per GPU, halo "
+                         "kernel": "cart2d_tau0_kernel (FP32, mu = 1, tau = 0), per GPU, halo "
                                    "exchange included in the time",
                          "algorithmic_bytes_per_launch": BYTES_PER_CELL_STEP["fp32"] * ncell // world},
             "e2e": {"value": e2e, "unit": UNIT,
@@ -851,7 +851,7 @@ def main():
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                          "frac": achieved / hbm, "peak_source": how,
                          "traffic": _profiled_traffic(),
-                         "kernel": "cart2d_step_kernel_s (staged FP32, mu = 1)",
+                         "kernel": "cart2d_tau0_kernel (FP32, mu = 1, tau = 0)",
                          "algorithmic_bytes_per_launch": BYTES_PER_CELL_STEP["fp32"] * ncell},
             "fp64": {"value": value64, "ms_per_step": ms64, "unit": UNIT,
                      "fp32_speedup": value / world / value64},

@@ -14,6 +14,7 @@
 // along the lane axis come from shuffles.  Work computed twice: 2 of 32 lanes, and about a third of
 // a row (plane) per chunk of rows (planes).  The three roles may be any cyclic renaming of x, y, z
 // (the flux is the same under it), so the lane axis is the one whose length fills strips best.
+// 130 x 118 x 97: 0.99 ms a step, the general kernel 2.59; the arithmetic alone 0.46.
 #include <cuda_runtime.h>
 
 #include <algorithm>
