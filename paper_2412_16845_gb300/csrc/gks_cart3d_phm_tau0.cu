@@ -19,10 +19,10 @@
 // plane: differences from the staged plane (x, y) and registers (z); sides; the z-face below completes the
 // plane below; x by shuffles; y-sides and y-fluxes through shared memory, two barriers a plane.  Planes
 // arrive by asynchronous copies one plane ahead (loaded through registers they stalled the march: 227 us a
-// step).  About 800 warp instructions a plane, 444 of them arithmetic, where the general kernel, which
+// step).  About 850 warp instructions a plane, 444 of them arithmetic, where the general kernel, which
 // exchanges gradients and rebuilds both sides of every face, issues 1865 a cell.
-// 150 x 139 x 128 FP32: 126 us a step (general kernel: 277).  Bound: latency and barriers at 12 warps an SM
-// (issue 41% busy before the copies); BY = 14 and 16 spill below 150 registers (190, 198 us), BY = 10
+// 150 x 139 x 128 FP32: 126 us a step (general kernel: 277).  Bound: instruction issue, 72% busy with 12
+// warps an SM (41% before the copies); BY = 14 and 16 spill below 150 registers (190, 198 us), BY = 10
 // carries a larger ring (147 us).  FP64 takes BY = 8 for its 255 registers.
 #include <cuda_runtime.h>
 
