@@ -465,12 +465,12 @@ cudaError_t launch_adjoint_tau0(const CartGeom &g, const AdjointArgs &a, cudaStr
   p.flag = a.flag;
   p.wx0 = a.window[0]; p.wx1 = a.window[1]; p.wy0 = a.window[2]; p.wy1 = a.window[3];
   constexpr int smem = (int)sizeof(Stage);
+  static_assert(smem <= 48 * 1024, "more needs the kernel's limit raised");
   static int sms = 0;
   if (!sms) {
     int dev = 0, n = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(adjoint_tau0_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     sms = n > 0 ? n : 1;
   }
   // Rows a chunk (which computes two rows more): one wave of five CTAs per SM while that takes 40 rows or

@@ -19,6 +19,7 @@
 
 #include "gks_flux2.cuh"
 #include "gks_internal.h"
+#include "gks_shared_limit.h"
 #include "gks_tma.cuh"
 
 namespace gks {
@@ -1220,15 +1221,14 @@ constexpr int kWaves2 = 4;
 cudaError_t launch_staged2(const CartGeom &g, const Cart2DPackArgs &P, int wx0, int wx1, int wy0,
                            int wy1, cudaStream_t st) {
   const int smem = WARPS * (int)sizeof(WarpStage2);
+  static SharedLimit limit;
+  const cudaError_t e = limit.raise(smem, cart2d_step_kernel_s<false>, cart2d_step_kernel_s<true>);
+  if (e != cudaSuccess) return e;
   static int per_sm = 0, sms = 0;
   if (!per_sm) {
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(cart2d_step_kernel_s<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         smem);
-    cudaFuncSetAttribute(cart2d_step_kernel_s<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cart2d_step_kernel_s<false>, WARPS * 32,
                                                   smem);
     if (sms < 1) sms = 1;

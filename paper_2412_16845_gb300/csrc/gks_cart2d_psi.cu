@@ -11,6 +11,7 @@
 
 #include "gks_flux2.cuh"
 #include "gks_internal.h"
+#include "gks_shared_limit.h"
 #include "gks_tma.cuh"
 
 namespace gks {
@@ -1030,13 +1031,14 @@ bool psi_staged_supported(const CartGeom &g, const CartStepArgs &a) {
 
 cudaError_t launch_psi_staged(const CartGeom &g, const PsiPackArgs &P, cudaStream_t st) {
   const int smem = PWARPS * (int)sizeof(PWarpStage2);
+  static SharedLimit limit;
+  const cudaError_t e = limit.raise(smem, cart2d_psi_step_kernel_s);
+  if (e != cudaSuccess) return e;
   static int per_sm = 0, sms = 0;
   if (!per_sm) {
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(cart2d_psi_step_kernel_s, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cart2d_psi_step_kernel_s, PWARPS * 32,
                                                   smem);
     if (sms < 1) sms = 1;

@@ -21,6 +21,7 @@
 #include "gks_internal.h"
 #include "gks_pdl.cuh"
 #include "gks_rcp.cuh"
+#include "gks_shared_limit.h"
 #include "gks_tau0_2d.cuh"
 
 namespace gks {
@@ -257,14 +258,9 @@ cudaError_t launch_t(const CartGeom &g, const CartStepArgs &a, const SmallPlan &
   const int grid = p.tiles_x * ((g.ny + pl.th - 1) / pl.th);
   constexpr int smem = N * NF * (int)sizeof(T);
   auto kern = a.limiter ? cart2d_small_kernel<T, true> : cart2d_small_kernel<T, false>;
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(cart2d_small_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         smem);
-    cudaFuncSetAttribute(cart2d_small_kernel<T, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         smem);
-    attr = true;
-  }
+  static SharedLimit limit;
+  const cudaError_t e = limit.raise(smem, cart2d_small_kernel<T, true>, cart2d_small_kernel<T, false>);
+  if (e != cudaSuccess) return e;
   return launch_pdl(kern, grid, NT<T>, smem, st, p);
 }
 

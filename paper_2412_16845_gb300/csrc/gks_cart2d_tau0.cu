@@ -659,12 +659,7 @@ cudaError_t launch_f32(const CartGeom &g, const CartStepArgs &a, cudaStream_t st
   static const K kern[2][2] = {{cart2d_tau0_kernel<false, false>, cart2d_tau0_kernel<false, true>},
                                {cart2d_tau0_kernel<true, false>, cart2d_tau0_kernel<true, true>}};
   constexpr int smem = (int)sizeof(Stage);
-  static bool attr = false;
-  if (!attr) {
-    for (int i = 0; i < 4; ++i)
-      cudaFuncSetAttribute(kern[i / 2][i % 2], cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    attr = true;
-  }
+  static_assert(smem <= 48 * 1024, "more needs the kernels' limit raised");
   const int sms = sm_count();
   const int wrows = p.wy1 - p.wy0, strips = (p.wx1 - p.wx0 + W - 1) / W;
   const int nw = std::min(WARPS, strips);

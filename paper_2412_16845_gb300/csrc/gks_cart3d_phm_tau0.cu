@@ -32,6 +32,7 @@
 #include "gks_internal.h"
 #include "gks_pdl.cuh"
 #include "gks_rcp.cuh"
+#include "gks_shared_limit.h"
 
 namespace gks {
 namespace {
@@ -420,6 +421,9 @@ cudaError_t launch_t(const CartGeom &g, const CartStepArgs &a, double chi, doubl
   p.pitch = g.pitch; p.plane = g.plane; p.cstride = g.cstride;
   p.flag = a.flag;
   constexpr int smem = (int)sizeof(Smem<T>);
+  static SharedLimit limit;
+  const cudaError_t e = limit.raise(smem, cart3d_phm_tau0_kernel<T, true>, cart3d_phm_tau0_kernel<T, false>);
+  if (e != cudaSuccess) return e;
   static int res[2] = {0, 0};
   auto kern = a.limiter ? cart3d_phm_tau0_kernel<T, true> : cart3d_phm_tau0_kernel<T, false>;
   int &resident = res[a.limiter ? 1 : 0];
@@ -427,7 +431,6 @@ cudaError_t launch_t(const CartGeom &g, const CartStepArgs &a, double chi, doubl
     int dev = 0, sms = 0, per = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, NTH, smem);
     resident = sms * (per > 0 ? per : 1);
   }

@@ -30,6 +30,7 @@
 #include <cuda_runtime.h>
 
 #include "gks_internal.h"
+#include "gks_shared_limit.h"
 #include "gks_side3.cuh"
 #include "gks_tma.cuh"
 
@@ -705,11 +706,9 @@ cudaError_t launch_cart3d_side(const CartGeom &g, const CartStepArgs &a, cudaStr
   }
   const int gx = (g.nx + TCOLS - 1) / TCOLS, gy = (g.ny + NWO - 1) / NWO;
   const int smem = (int)sizeof(SideSmem);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(cart3d_side_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    attr = true;
-  }
+  static SharedLimit limit;
+  const cudaError_t e = limit.raise(smem, cart3d_side_kernel);
+  if (e != cudaSuccess) return e;
   static int sms = 0;
   if (!sms) {
     int dev = 0;

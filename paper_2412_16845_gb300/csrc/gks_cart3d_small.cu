@@ -16,6 +16,7 @@
 #include "gks_pdl.cuh"
 #include "gks_pair3.cuh"
 #include "gks_rcp.cuh"
+#include "gks_shared_limit.h"
 
 namespace gks {
 namespace {
@@ -240,14 +241,10 @@ cudaError_t launch_t(const CartGeom &g, const CartStepArgs &a, cudaStream_t st) 
   p.tiles[0] = (g.nx + L::B0 - 1) / L::B0;
   p.tiles[1] = (g.ny + L::B1 - 1) / L::B1;
   const int grid = p.tiles[0] * p.tiles[1] * ((g.nz + L::B2 - 1) / L::B2);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(cart3d_small_kernel<T, I, true>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    cudaFuncSetAttribute(cart3d_small_kernel<T, I, false>,
-                         cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    attr = true;
-  }
+  static SharedLimit limit;
+  const cudaError_t e =
+      limit.raise(smem, cart3d_small_kernel<T, I, true>, cart3d_small_kernel<T, I, false>);
+  if (e != cudaSuccess) return e;
   auto kern = a.limiter ? cart3d_small_kernel<T, I, true> : cart3d_small_kernel<T, I, false>;
   return launch_pdl(kern, grid, L::NT, smem, st, p);
 }

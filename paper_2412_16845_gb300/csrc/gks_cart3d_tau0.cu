@@ -16,6 +16,7 @@
 #include "gks_pdl.cuh"
 #include "gks_pair3.cuh"
 #include "gks_rcp.cuh"
+#include "gks_shared_limit.h"
 #include "gks_tma.cuh"
 
 namespace gks {
@@ -599,11 +600,9 @@ cudaError_t launch_cart3d_tau0(const CartGeom &g, const CartStepArgs &a, cudaStr
     for (int q = 0; q < 2; ++q) p.k[A][q] = make_pair_k<float>(a.C, g.h, a.c, A, q);
   const int gx = (g.nx + TCOLS - 1) / TCOLS, gy = (g.ny + NWO - 1) / NWO;
   const int smem = (int)sizeof(Smem);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(cart3d_tau0_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    attr = true;
-  }
+  static SharedLimit limit;
+  const cudaError_t e = limit.raise(smem, cart3d_tau0_kernel);
+  if (e != cudaSuccess) return e;
   static int sms = 0;
   if (!sms) {
     int dev = 0;

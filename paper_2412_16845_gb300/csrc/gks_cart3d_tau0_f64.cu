@@ -24,6 +24,7 @@
 #include "gks_internal.h"
 #include "gks_pair3.cuh"
 #include "gks_rcp.cuh"
+#include "gks_shared_limit.h"
 
 namespace gks {
 namespace {
@@ -286,15 +287,15 @@ bool cart3d_tau0_f64_supported(const CartStepArgs &a) {
 }
 
 cudaError_t launch_cart3d_tau0_f64(const CartGeom &g, const CartStepArgs &a, cudaStream_t st) {
+  static SharedLimit limit;
+  const cudaError_t e = limit.raise(WARPS * MAXR * NST * 32 * 8, cart3d_tau0_f64_kernel<false>,
+                                    cart3d_tau0_f64_kernel<true>);
+  if (e != cudaSuccess) return e;
   static int sms = 0;
   if (!sms) {
     int dev = 0, n = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
-    cudaFuncSetAttribute(cart3d_tau0_f64_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         WARPS * MAXR * NST * 32 * 8);
-    cudaFuncSetAttribute(cart3d_tau0_f64_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         WARPS * MAXR * NST * 32 * 8);
     sms = n > 0 ? n : 1;
   }
   Args p;
