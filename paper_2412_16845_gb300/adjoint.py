@@ -40,6 +40,8 @@ class DesignProblem:
         self.N = int(nsteps if nsteps is not None else w.steps)
         self.K = int(checkpoint_every or max(1, int(round(math.sqrt(self.N)))))
         self.stream = stream if stream is not None else torch.cuda.current_stream()
+        if not isinstance(self.stream, torch.cuda.Stream):      # an object with the stream's handle
+            self.stream = torch.cuda.ExternalStream(self.stream.cuda_stream)
         self.base_eps = np.array(w.eps, dtype=np.float64)
         self.design = np.asarray(w.design, dtype=np.int64)
         mu = np.ones_like(self.base_eps) if w.mu is None else np.asarray(w.mu, dtype=np.float64)
@@ -54,7 +56,8 @@ class DesignProblem:
         self.elems, _ = gks_state_layout(self.ctx)
         self.dtype = torch.float64 if precision == "fp64" else torch.float32
         # V^0 stays on the device; each forward() restarts from it
-        self.init = self._buf()
+        with torch.cuda.stream(self.stream):
+            self.init = self._buf()
         gks_copy_state(self.ctx, self.init.data_ptr())
         # a design update rewrites eps only on the design's bounding box
         self.dbox, self.dbox_index, cells = design_box(self.design, w.n[0])
@@ -96,6 +99,8 @@ class DesignProblem:
         x0, x1, y0, y1 = max(a[0], b[0]), min(a[1], b[1]), max(a[2], b[2]), min(a[3], b[3])
         return (x0, x1, y0, y1) if x0 < x1 and y0 < y1 else None
 
+    # Device buffers belong to the problem's stream, on which the kernels use them: they are made, filled
+    # and given back in its order, whatever the caller's current stream is.
     def _buf(self):
         return self.torch.empty(self.elems, dtype=self.dtype, device="cuda")
 
@@ -117,6 +122,10 @@ class DesignProblem:
 
     def forward(self, eps_design, keep_checkpoints=True):
         """J(eps_design); keeps the checkpoints for a following backward()."""
+        with self.torch.cuda.stream(self.stream):
+            return self._forward(eps_design, keep_checkpoints)
+
+    def _forward(self, eps_design, keep_checkpoints):
         self.set_design(eps_design)
         gks_load_state(self.ctx, self.init.data_ptr(), 0)
         gks_reset_objective(self.ctx)
@@ -138,10 +147,19 @@ class DesignProblem:
         return J
 
     def backward(self):
-        """dJ/d eps over the design cells (device float64 tensor), after forward()."""
-        torch = self.torch
+        """dJ/d eps over the design cells (device float64 tensor), after forward().  The caller's current
+        stream waits for it."""
         if self.checkpoints is None:
             raise RuntimeError("forward() with keep_checkpoints=True must come first")
+        caller = self.torch.cuda.current_stream()
+        with self.torch.cuda.stream(self.stream):
+            grad = self._backward()
+        caller.wait_stream(self.stream)
+        grad.record_stream(caller)
+        return grad
+
+    def _backward(self):
+        torch = self.torch
         # (zero where lambda is never computed; the pool's entries off the recomputed windows are
         # never read into a result, but have to be finite)
         lam, lam2 = self._zeros(), self._zeros()

@@ -21,6 +21,8 @@ std::map<std::pair<int, const void *>, int> shared_limit;
 std::string launched;                 // names of the kernels launched, one a line
 int device = 0;
 int allocations_left = -1;            // -1: never fails
+std::string gives_up;                 // a launch of a kernel of this name runs out of its bounded waits ...
+bool gave_up = false;                 // ... and leaves 2 in the context's flag, the one int the host reads
 cudaError_t last = cudaSuccess;
 struct { dim3 grid, block; size_t smem; cudaStream_t st; } pushed;
 
@@ -29,6 +31,7 @@ cudaError_t launch(const void *f, size_t smem) {
   const size_t limit = it == shared_limit.end() ? 48 * 1024 : (size_t)it->second;
   if (smem > limit) return last = cudaErrorInvalidValue;
   launched += kernels()[f] + "\n";
+  if (!gives_up.empty() && kernels()[f].find(gives_up) != std::string::npos) gave_up = true;
   return cudaSuccess;
 }
 
@@ -51,6 +54,7 @@ void fake_set_device(int d) { device = d; }
 void fake_fail_allocation(int after) { allocations_left = after; }
 const char *fake_launched() { return launched.c_str(); }
 void fake_clear() { launched.clear(); }
+void fake_give_up(const char *kernel) { gives_up = kernel; gave_up = false; }
 
 // registration and <<<>>>
 void **__cudaRegisterFatBinary(void *) { static void *h; return &h; }
@@ -108,8 +112,9 @@ cudaError_t cudaMallocAsync(void **p, size_t n, cudaStream_t) {
   return *p ? cudaSuccess : cudaErrorMemoryAllocation;
 }
 cudaError_t cudaFreeAsync(void *p, cudaStream_t) { free(p); return cudaSuccess; }
-cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t) {
+cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind kind, cudaStream_t) {
   memmove(d, s, n);
+  if (gave_up && kind == cudaMemcpyDeviceToHost && n == sizeof(int)) *(int *)d = 2;
   return cudaSuccess;
 }
 cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t) { memset(d, v, n); return cudaSuccess; }

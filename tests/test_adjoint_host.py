@@ -1,0 +1,38 @@
+"""The host side of DesignProblem without a GPU (tests/fake_cuda.py): streams, errors, windows."""
+import numpy as np
+import pytest
+
+from paper_2412_16845_gb300 import workloads as wl
+from tests.fake_cuda import _fake_library, fake, fake_torch  # noqa: F401
+
+
+def _workload(nx=40, ny=32, bc=("nrbc",) * 4, steps=20, design=((8, 16), (6, 14)), probe=((24, 27), (15, 18))):
+    def cells(b):
+        return (np.arange(*b[1])[:, None] * nx + np.arange(*b[0])[None, :]).ravel()
+    return wl.CartWorkload(name="design", dim=2, n=(nx, ny), lo=(0.0, 0.0), hi=(1.0, ny / nx), bc=bc, cfl=0.5,
+                           steps=steps, eps=np.full(nx * ny, 2.0), mu=None, fields0=np.zeros((3, nx * ny)),
+                           jz_mask=None, src=None, c_lattice=1.0, probe=cells(probe), design=cells(design))
+
+
+def _problem(w, **kw):
+    from paper_2412_16845_gb300.adjoint import DesignProblem
+    return DesignProblem(w, **kw)
+
+
+@pytest.mark.parametrize("own", [False, True])
+def test_buffers_live_on_the_problems_stream(fake_torch, own):
+    """Every buffer that kernels on the problem's stream write is made (and filled) on that stream, and the
+    caller's stream waits for the gradient, whichever stream is current at each call."""
+    t = fake_torch
+    side = t.Stream(t, "side")
+    p = _problem(_workload(), **({"stream": side} if own else {}))
+    mine = "side" if own else "caller"
+    for name in ("caller", "another"):
+        t.current = t.Stream(t, name)
+        p.forward(p.base_eps[p.design])
+        g = p.backward()
+        assert set(t.made) == {mine}, t.made
+        assert t.current.name == name
+        if name != mine:
+            assert (name, mine) in t.waits and name in g.streams
+    p.close()
