@@ -16,7 +16,7 @@ import numpy as np
 
 from .gks import (GKSSolver, gks_adjoint_seed, gks_adjoint_step_window, gks_copy_state,
                   gks_load_state, gks_objective, gks_reset_objective, gks_set_materials_box,
-                  gks_set_objective, gks_state_layout, gks_step_state_window)
+                  gks_set_objective, gks_state_layout, gks_step_state_window, gks_sync)
 
 
 def design_box(design, nx):
@@ -147,8 +147,8 @@ class DesignProblem:
         return J
 
     def backward(self):
-        """dJ/d eps over the design cells (device float64 tensor), after forward().  The caller's current
-        stream waits for it."""
+        """dJ/d eps over the design cells (device float64 tensor), after forward(); complete on return.
+        GksError (GKS_E_TIMEOUT) if a kernel's bounded wait ran out."""
         if self.checkpoints is None:
             raise RuntimeError("forward() with keep_checkpoints=True must come first")
         caller = self.torch.cuda.current_stream()
@@ -185,6 +185,9 @@ class DesignProblem:
                     gks_adjoint_step_window(ctx, ptrs[n - s], ptrs[n - s + 1], lam_ptr, lam2_ptr,
                                             grad_ptr, n >= 1, *win)
                 lam_ptr, lam2_ptr = lam2_ptr, lam_ptr
+        # waits for the stream: the recomputed steps and the lambda march have bounded waits, and one that
+        # ran out has to be an error here, not a wrong gradient now and an error of the next forward()
+        gks_sync(ctx)
         del pool
         return grad
 

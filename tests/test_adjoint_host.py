@@ -36,3 +36,16 @@ def test_buffers_live_on_the_problems_stream(fake_torch, own):
         if name != mine:
             assert (name, mine) in t.waits and name in g.streams
     p.close()
+
+
+@pytest.mark.parametrize("kernel", [b"adjoint_tau0_kernel", b"cart2d_tau0_kernel"])
+def test_a_wait_that_ran_out_in_backward_is_an_error(fake, fake_torch, kernel):
+    """The lambda march and the recomputed steps have bounded waits; a wrong gradient is not returned."""
+    from paper_2412_16845_gb300 import gks
+    p = _problem(_workload())
+    p.forward(p.base_eps[p.design])
+    fake.give_up(kernel)
+    with pytest.raises(gks.GksError) as e:
+        p.backward()
+    assert e.value.status == gks.GKS_E_TIMEOUT
+    p.close()
