@@ -72,7 +72,7 @@ class DesignProblem:
         nx, ny = w.n
         self.nx, self.ny = nx, ny
         self.per = (w.bc[0] == "periodic", w.bc[2] == "periodic")
-        self.pbox = self._box(w.probe)
+        self.pbox = self._box(w.probe) if len(w.probe) else None     # an empty probe: J = 0
         self.cbox = self._widen(self._box(np.concatenate([self.design,
                                                           np.asarray(w.probe, dtype=np.int64)])), 2)
 
@@ -94,6 +94,8 @@ class DesignProblem:
         """Where lambda^n is computed, or None: it is zero beyond two cells per step n .. N around the
         probe, and the steps below n carry only the cells within 2 n of the design region into the
         gradient."""
+        if self.pbox is None:
+            return None
         a = self._widen(self.pbox, 2 * (self.N - n))
         b = self._widen(self.dbox, 2 * n + 2)
         x0, x1, y0, y1 = max(a[0], b[0]), min(a[1], b[1]), max(a[2], b[2]), min(a[3], b[3])

@@ -49,3 +49,15 @@ def test_a_wait_that_ran_out_in_backward_is_an_error(fake, fake_torch, kernel):
         p.backward()
     assert e.value.status == gks.GKS_E_TIMEOUT
     p.close()
+
+
+@pytest.mark.parametrize("bc", [("nrbc",) * 4, ("periodic",) * 4])
+def test_an_empty_probe_has_a_zero_gradient(fake, fake_torch, bc):
+    """gks_set_objective takes an empty probe: J = 0, and no lambda acts anywhere."""
+    w = _workload(bc=bc)
+    w.probe = np.zeros(0, dtype=np.int64)
+    p = _problem(w)
+    J = p.forward(p.base_eps[p.design])
+    g = p.backward()
+    assert J == 0.0 and g.t.shape == (p.design.size,) and not g.t.any()
+    p.close()

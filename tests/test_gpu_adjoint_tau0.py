@@ -49,3 +49,14 @@ def test_gradient_on_another_stream():
         g = p.backward().cpu().numpy()
         p.close()
         assert J == J0 and np.array_equal(g, g0)
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+def test_an_empty_probe_has_a_zero_gradient(precision):
+    from paper_2412_16845_gb300.adjoint import DesignProblem
+    w = _design(40, 30, OPEN, 9, ((10, 20), (8, 15)), ((30, 31), (5, 6)))
+    w.probe = w.probe[:0]
+    p = DesignProblem(w, precision=precision, checkpoint_every=4)
+    J, g = p.value_and_grad(w.eps[w.design])
+    p.close()
+    assert J == 0.0 and g.size == w.design.size and not g.any()
