@@ -174,7 +174,8 @@ gks_status gks_step_window(gks_ctx *ctx, int64_t n_steps, int64_t x0, int64_t x1
  * the window [x0, x1) x [y0, y1) of a 2-D Cartesian grid, as step number `step` (the source is taken
  * at t0 + step dt).  The context's own state, time and step counter stay.  Entries of dst outside the
  * window are left as they are or hold stale values; the window's cells need src on the window
- * widened by two cells.  Asynchronous. */
+ * widened by two cells and finite values elsewhere.  States that start on a multiple of 16 bytes suit every
+ * kernel; others run a slower one or, if no kernel takes them, are refused.  Asynchronous. */
 gks_status gks_step_state_window(gks_ctx *ctx, const void *src, void *dst, int64_t step, int64_t x0,
                                  int64_t x1, int64_t y0, int64_t y1);
 
@@ -234,7 +235,8 @@ gks_status gks_adjoint_seed(gks_ctx *ctx, const void *state, void *adj);
  * grad_eps[k] += dV^{n+1}/d eps_{design[k]} . adj_in, with V^{n+1} = L(eps) V^n + s^n.
  * state_n = V^n, state_np1 = V^{n+1} (device, internal layout; needed on the design cells and
  * the probe), adj_in = lambda^{n+1}, adj_out = lambda^n (distinct device buffers),
- * grad_eps: device [nd] doubles.  2-D TM, mu = 1.  Asynchronous. */
+ * grad_eps: device [nd] doubles.  2-D TM, mu = 1.  adj_in and adj_out start on multiples of two values
+ * (16 bytes suit every kernel).  Asynchronous. */
 gks_status gks_adjoint_step(gks_ctx *ctx, const void *state_n, const void *state_np1,
                             const void *adj_in, void *adj_out, double *grad_eps,
                             int32_t add_probe);

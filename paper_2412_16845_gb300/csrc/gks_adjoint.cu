@@ -611,6 +611,8 @@ cudaError_t adjoint_t(const CartGeom &g, const AdjointArgs &a, cudaStream_t st) 
   cudaError_t e;
   if (tau0 && sizeof(T) == 4) {
     e = launch_adjoint_tau0(g, a, st);
+  } else if (!aligned(a.lam_in, 2 * sizeof(T)) || !aligned(a.lam_out, 2 * sizeof(T))) {
+    return cudaErrorInvalidValue;                     // it loads and stores pairs
   } else {
     adjoint_lambda_kernel<T><<<grid, AWARPS * 32, 0, st>>>(p, nstrips, rows);
     e = cudaGetLastError();

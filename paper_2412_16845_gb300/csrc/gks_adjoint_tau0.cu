@@ -444,7 +444,7 @@ Axis make_adj_axis(const double C[5], double c, double hn, double ht, double sig
 bool adjoint_tau0_supported(const CartGeom &g, const AdjointArgs &a) {
   if (a.C[1] != 0.0 || a.C[3] != 0.0 || a.C[4] != 0.0 || !(a.C[0] > 0.0) || !a.eps_normal) return false;
   if (g.periodic[1] && g.ny < 2) return false;        // the staged rows wrap by one period
-  return tensor_map_encoder() != nullptr;
+  return aligned(a.lam_in, 16) && tensor_map_encoder() != nullptr;
 }
 
 cudaError_t launch_adjoint_post_tau0(const CartGeom &g, const AdjointArgs &a, const int box[4],

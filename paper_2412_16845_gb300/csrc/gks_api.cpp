@@ -749,6 +749,8 @@ gks_status gks_step_state_window(gks_ctx *ctx, const void *src, void *dst, int64
     return fail(ctx, GKS_E_UNSUPPORTED, "windowed steps need a 2-D Cartesian grid");
   if (ctx->phm) return fail(ctx, GKS_E_UNSUPPORTED, "windowed steps do not cover divergence cleaning");
   if (!src || !dst || src == dst || step < 0) return fail(ctx, GKS_E_ARG, "src / dst / step");
+  if (!gks::aligned(src, ctx->esize) || !gks::aligned(dst, ctx->esize))
+    return fail(ctx, GKS_E_ARG, "src / dst alignment");
   if (x0 < 0 || y0 < 0 || x1 > ctx->g.nx || y1 > ctx->g.ny || x0 >= x1 || y0 >= y1)
     return fail(ctx, GKS_E_ARG, "window outside the grid or empty");
   const int win[4] = {(int)x0, (int)x1, (int)y0, (int)y1};
@@ -958,6 +960,8 @@ gks_status gks_adjoint_step_window(gks_ctx *ctx, const void *state_n, const void
     if (ctx->g.pec[k])
       return fail(ctx, GKS_E_UNSUPPORTED, "the adjoint supports periodic and non-reflecting sides only");
   if (!adj_in || !adj_out || adj_in == adj_out) return fail(ctx, GKS_E_ARG, "adj_in / adj_out");
+  if (!gks::aligned(adj_in, ctx->esize) || !gks::aligned(adj_out, ctx->esize))
+    return fail(ctx, GKS_E_ARG, "adj_in / adj_out alignment");
   if (ctx->nd > 0 && (!grad_eps || !state_n || !state_np1))
     return fail(ctx, GKS_E_ARG, "the eps-gradient needs both states and grad_eps");
   if (add_probe && ctx->np > 0 && !state_n) return fail(ctx, GKS_E_ARG, "state_n is NULL");

@@ -1210,7 +1210,7 @@ Coef<T> make_coef(const double C[5], double h, double c) {
 bool staged2_supported(const CartGeom &g, const CartStepArgs &a) {
   if (a.mu || a.limiter || g.periodic[0]) return false;
   if (g.periodic[1] && g.ny < 2) return false;
-  return tensor_map_encoder() != nullptr;
+  return aligned(a.V, 16) && tensor_map_encoder() != nullptr;
 }
 
 // Staged launch over the window's columns [wx0, wx1) (strips of W2 columns) and rows [wy0, wy1):
@@ -1299,6 +1299,7 @@ cudaError_t launch_t(const CartGeom &g, const CartStepArgs &a, cudaStream_t st) 
   // PEC walls and the limiter get their own instantiations: without them the mirror
   // bookkeeping and the limiter fold away
   const bool pec = g.pec[0] || g.pec[1] || g.pec[2] || g.pec[3];
+  const bool pairs = aligned(a.V, 2 * sizeof(T)) && aligned(a.Vout, 2 * sizeof(T));
   using K = void (*)(const Cart2DKernelArgs<T>, int, int, int, int, int);
   static const K kern[2][2][2] = {   // [mu][pec][limiter]
       {{cart2d_step_kernel<T, false, false, false>, cart2d_step_kernel<T, false, false, true>},
@@ -1312,6 +1313,7 @@ cudaError_t launch_t(const CartGeom &g, const CartStepArgs &a, cudaStream_t st) 
       P.fx = make_face_kp(p.fx);
       P.fy = make_face_kp(p.fy);
       if (staged2_supported(g, a)) return launch_staged2(g, P, wx0, wx1, wy0, wy1, st);
+      if (!pairs) return cudaErrorInvalidValue;
       using KP = void (*)(const Cart2DPackArgs, int, int, int, int, int);
       static const KP kp[2][2] = {{cart2d_step_kernel_p<false, false>,
                                    cart2d_step_kernel_p<false, true>},
@@ -1322,6 +1324,7 @@ cudaError_t launch_t(const CartGeom &g, const CartStepArgs &a, cudaStream_t st) 
       return cudaGetLastError();
     }
   }
+  if (!pairs) return cudaErrorInvalidValue;
   kern[a.mu ? 1 : 0][pec ? 1 : 0][a.limiter ? 1 : 0]<<<grid, WARPS * 32, 0, st>>>(
       p, nstrips, rows, strip0, wy0, wy1);
   return cudaGetLastError();

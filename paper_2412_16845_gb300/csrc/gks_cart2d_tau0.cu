@@ -730,7 +730,7 @@ bool cart2d_tau0_supported(const CartGeom &g, const CartStepArgs &a, bool fp64) 
     return false;
   if (fp64) return true;
   if (g.periodic[1] && g.ny < 2) return false;        // FP32: the staged rows wrap by one period
-  return tensor_map_encoder() != nullptr;
+  return aligned(a.V, 16) && tensor_map_encoder() != nullptr;
 }
 
 cudaError_t launch_cart2d_tau0(const CartGeom &g, const CartStepArgs &a, bool fp64,

@@ -15,6 +15,10 @@ namespace gks {
 // time tau (tau = 0: the tau -> 0 limit of Sec. 4.1).
 void time_coefficients(double dt, double tau, double C[5]);
 
+// Whether p lies on a multiple of `bytes`.  A context's own states lie on 256 bytes; a caller's may be a
+// slice of anything: tensor copies need 16 bytes, kernels that load pairs two values, the rest one.
+inline bool aligned(const void *p, size_t bytes) { return reinterpret_cast<uintptr_t>(p) % bytes == 0; }
+
 // Cartesian grid geometry and state layout.  Fields are stored structure-of-arrays,
 // [ncomp][nz][ny][pitch] with x fastest; pitch is nx rounded up to a multiple of 32 elements
 // (128 B rows in FP32) so that every row starts 128-byte aligned.
@@ -31,8 +35,8 @@ struct CartGeom {
 
 // Arguments of one Cartesian step launch (precision-independent; kernels cast).
 struct CartStepArgs {
-  const void *V;        // state at t^n
-  void *Vout;           // state at t^{n+1}
+  const void *V = nullptr;  // state at t^n
+  void *Vout = nullptr;     // state at t^{n+1}
   const void *eps;      // [nz][ny][pitch]
   const void *mu;       // same layout, or nullptr (mu = 1)
   const void *src;      // J_z mask, same layout, or nullptr

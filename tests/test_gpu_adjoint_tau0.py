@@ -60,3 +60,27 @@ def test_an_empty_probe_has_a_zero_gradient(precision):
     J, g = p.value_and_grad(w.eps[w.design])
     p.close()
     assert J == 0.0 and g.size == w.design.size and not g.any()
+
+
+def test_a_callers_states_between_16_byte_boundaries():
+    """FP32 states 8 bytes past a 16-byte boundary: the adjoint and the step run without tensor copies and
+    agree with the aligned calls to rounding."""
+    import torch
+    from paper_2412_16845_gb300 import gks
+    w = _design(70, 40, OPEN, 1, ((10, 20), (8, 15)), ((30, 31), (5, 6)))
+    s = gks.GKSSolver.from_workload(w, precision="fp32")
+    gks.gks_set_objective(s.ctx, None, None)
+    n, _ = gks.gks_state_layout(s.ctx)
+    x = torch.zeros(n, device="cuda")
+    gks.gks_copy_state(s.ctx, x.data_ptr())
+    out = []
+    for off in (0, 2):
+        src, dst, lam = (torch.zeros(n + 4, device="cuda")[off:off + n] for _ in range(3))
+        src.copy_(x)
+        gks.gks_step_state_window(s.ctx, src.data_ptr(), dst.data_ptr(), 0, 0, 70, 0, 40)
+        gks.gks_adjoint_step(s.ctx, None, None, src.data_ptr(), lam.data_ptr(), None, False)
+        gks.gks_sync(s.ctx)
+        out.append((dst.clone(), lam.clone()))
+    s.close()
+    for a, b in zip(out[0], out[1]):
+        assert float((a - b).norm()) <= 2e-5 * float(a.norm()) and float(a.norm()) > 0

@@ -49,3 +49,67 @@ def test_a_second_device_gets_its_shared_memory(fake, n, bc, limiter, phm, kappa
         names = fake.launched()
         s.close()
         assert names and all(kernel in k for k in names), names
+
+
+def _states(w, precision, *offsets):
+    """Host buffers for states of w that start `offset` bytes past a 16-byte boundary."""
+    from paper_2412_16845_gb300 import gks
+    s = GKSSolver.from_workload(w, precision=precision)
+    _, nbytes = gks.gks_state_layout(s.ctx)
+    s.close()
+    bufs = [np.zeros(nbytes + 64, dtype=np.uint8) for _ in offsets]
+    return bufs, [(b.ctypes.data + 31) // 16 * 16 + o for b, o in zip(bufs, offsets)]
+
+
+# kernels that copy rows by tensor maps need 16 bytes, those that load pairs need a pair, the rest a value
+@pytest.mark.parametrize("precision,kappa,bc,src,dst,kernel", [
+    ("fp32", 0.0, "nnnn", 0, 4, "cart2d_tau0_kernel"),
+    ("fp32", 0.0, "nnnn", 8, 8, "cart2d_step_kernel_p"),
+    ("fp32", 0.05, "nnnn", 0, 4, "cart2d_step_kernel_s"),
+    ("fp32", 0.05, "nnnn", 8, 8, "cart2d_step_kernel_p"),
+    ("fp32", 0.05, "ppnn", 4, 0, None),
+    ("fp32", 0.05, "ppnn", 0, 4, None),
+    ("fp64", 0.0, "nnnn", 8, 8, "cart2d_tau0_f64_kernel"),
+    ("fp64", 0.05, "nnnn", 8, 0, None),
+    ("fp64", 0.05, "nnnn", 0, 0, "cart2d_step_kernel"),
+])
+def test_a_callers_state_goes_to_a_kernel_that_takes_its_alignment(fake, precision, kappa, bc, src, dst, kernel):
+    from paper_2412_16845_gb300 import gks
+    w = _grid((40, 30), bc)
+    keep, (p, q) = _states(w, precision, src, dst)
+    s = GKSSolver.from_workload(w, precision=precision, kappa=kappa)
+    fake.launched()
+    if kernel is None:
+        with pytest.raises(gks.GksError):
+            gks.gks_step_state_window(s.ctx, p, q, 0, 0, 40, 0, 30)
+        assert not fake.launched()
+    else:
+        gks.gks_step_state_window(s.ctx, p, q, 0, 0, 40, 0, 30)
+        assert [kernel + "I" in k or kernel + "E" in k for k in fake.launched()] == [True]
+    s.close()
+
+
+@pytest.mark.parametrize("precision,kappa,lam,out,kernel", [
+    ("fp32", 0.0, 0, 4, "adjoint_tau0_kernel"),
+    ("fp32", 0.0, 8, 8, "adjoint_lambda_kernel"),     # accepted before the march by tensor copies came
+    ("fp32", 0.05, 8, 0, "adjoint_lambda_kernel"),
+    ("fp32", 0.05, 0, 4, None),
+    ("fp64", 0.0, 8, 0, None),
+    ("fp64", 0.0, 0, 0, "adjoint_lambda_kernel"),
+])
+def test_a_callers_lambda_goes_to_a_kernel_that_takes_its_alignment(fake, precision, kappa, lam, out, kernel):
+    from paper_2412_16845_gb300 import gks
+    w = _grid((40, 30), "nnpp")
+    keep, (p, q) = _states(w, precision, lam, out)
+    s = GKSSolver.from_workload(w, precision=precision, kappa=kappa)
+    gks.gks_set_objective(s.ctx, None, None)
+    fake.launched()
+    if kernel is None:
+        with pytest.raises(gks.GksError):
+            gks.gks_adjoint_step(s.ctx, None, None, p, q, None, False)
+        assert not fake.launched()
+    else:
+        gks.gks_adjoint_step(s.ctx, None, None, p, q, None, False)
+        names = fake.launched()
+        assert len(names) >= 1 and kernel in names[0], names
+    s.close()
