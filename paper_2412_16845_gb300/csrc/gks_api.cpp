@@ -479,6 +479,7 @@ gks_status gks_set_materials(gks_ctx *ctx, const double *eps, const double *mu) 
   const double cmax = std::fmax(cleaning_speed(ctx), 1.0 / std::sqrt(mu ? em.least() : e.least()));
   const bool normal = normal_eps(e.least()) && normal_eps(e.most());
   gks_status s;
+  ctx->eps_normal = ctx->eps_normal && normal;   // before the upload: a call that fails leaves either eps
   if ((s = upload_cells(ctx, eps, 1, ctx->eps)) != GKS_OK) return s;
   if (mu) {
     if (!ctx->mu) {
@@ -511,11 +512,11 @@ gks_status gks_set_materials_box(gks_ctx *ctx, int64_t x0, int64_t x1, int64_t y
       return fail(ctx, GKS_E_ARG, "eps must be finite and > 0 (box entry " + std::to_string(i) + ")");
     normal = normal && normal_eps(eps_box[i]);
   }
+  ctx->eps_normal = normal;                      // before the upload, as in gks_set_materials
   GKS_CUDA(cudaMemcpyAsync(ctx->staging, eps_box, sizeof(double) * (size_t)n,
                            cudaMemcpyHostToDevice, ctx->st));
   GKS_CUDA(gks::launch_box_to_cart(ctx->staging, ctx->eps, (int)x0, (int)(x1 - x0), (int)y0,
                                    (int)(y1 - y0), ctx->g.pitch, ctx->fp64, ctx->st));
-  ctx->eps_normal = normal;
   return GKS_OK;
 }
 

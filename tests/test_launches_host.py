@@ -113,3 +113,26 @@ def test_a_callers_lambda_goes_to_a_kernel_that_takes_its_alignment(fake, precis
         names = fake.launched()
         assert len(names) >= 1 and kernel in names[0], names
     s.close()
+
+
+def test_a_failed_change_of_materials_keeps_extreme_permittivities_off_the_fast_reciprocals(fake):
+    """set_materials that uploads eps and then finds no memory for mu: the context holds the new eps."""
+    from paper_2412_16845_gb300 import gks
+    w = _grid((40, 30), "nnnn")
+    s = GKSSolver.from_workload(w, precision="fp32")
+    fake.launched()
+    s.step(1)
+    assert "cart2d_small_kernel" in fake.launched()[0]
+    fake.fail_allocation(0)
+    with pytest.raises(gks.GksError):
+        s.set_materials(np.full(1200, 1e-35), np.ones(1200))
+    fake.fail_allocation(-1)
+    fake.dll.cudaGetLastError()                       # the runtime's own record of the failed allocation
+    fake.launched()
+    s.step(1)
+    assert "cart2d_step_kernel_s" in fake.launched()[0]
+    s.set_materials(np.ones(1200))
+    fake.launched()
+    s.step(1)
+    assert "cart2d_small_kernel" in fake.launched()[0]
+    s.close()
