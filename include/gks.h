@@ -164,8 +164,8 @@ gks_status gks_step(gks_ctx *ctx, int64_t n_steps);
 /* Enqueue n_steps steps that advance only the cells of the window [x0, x1) x [y0, y1) (2-D
  * Cartesian grids).  Cells outside the window keep stale values, which act on the window's
  * cells after one step through the stencil (radius two cells): after k windowed steps only the
- * cells at least 2k cells inside the window are exact.  Used to recompute a region's domain of
- * dependence from a checkpoint (adjoint).  Time and step counter advance as in gks_step; the
+ * cells at least 2k cells inside the window are exact, and repeat the bits of whole steps.  Used to
+ * recompute a region's domain of dependence from a checkpoint (adjoint).  Time and step counter advance as in gks_step; the
  * probe objective is not accumulated. */
 gks_status gks_step_window(gks_ctx *ctx, int64_t n_steps, int64_t x0, int64_t x1, int64_t y0,
                            int64_t y1);

@@ -649,22 +649,31 @@ gks::CartStepArgs step_args(const gks_ctx *ctx, const int win[4]) {
   return a;
 }
 
+// 2-D grids too small to fill the GPU take cart2d_small_kernel for every step, whole steps and steps over
+// a window alike, so that a recomputed state repeats the bits of the forward pass.
+bool may_be_small2(const gks_ctx *ctx, const gks::CartStepArgs &a) {
+  return ctx->kind == GKS_CARTESIAN && ctx->dim == 2 && !ctx->phm &&
+         gks::cart2d_tau0_supported(ctx->g, a, ctx->fp64);
+}
+
+gks::SmallPlan small_plan2(gks_ctx *ctx, int most) {
+  if (!ctx->have2[most]) {
+    ctx->plan2[most] = gks::cart2d_small_plan(ctx->g, ctx->fp64, most);
+    ctx->have2[most] = true;
+  }
+  return ctx->plan2[most];
+}
+
 // Advance n_steps over the window [x0, x1) x [y0, y1) (2-D) or the whole mesh.
 gks_status step_impl(gks_ctx *ctx, int64_t n_steps, const int win[4], bool objective) {
   gks::CartStepArgs a = step_args(ctx, win);
-  // windowed steps (objective = false) march: their windows are recomputed step by step
-  const bool small2 = objective && ctx->kind == GKS_CARTESIAN && ctx->dim == 2 && !ctx->phm &&
-                      gks::cart2d_tau0_supported(ctx->g, a, ctx->fp64);
+  const bool small2 = may_be_small2(ctx, a);
   const bool small3 = ctx->kind == GKS_CARTESIAN && ctx->dim == 3 && !ctx->phm &&
                       gks::cart3d_tau0_f64_supported(a);
   const bool probe = objective && ctx->np > 0;       // needs the state after every step
-  auto plan2 = [ctx, probe](int64_t left) {
-    const int most = probe ? 1 : (int)std::min<int64_t>(left, gks::kSmallSteps);
-    if (!ctx->have2[most]) {
-      ctx->plan2[most] = gks::cart2d_small_plan(ctx->g, ctx->fp64, most);
-      ctx->have2[most] = true;
-    }
-    return ctx->plan2[most];
+  const bool whole = win[0] == 0 && win[1] == ctx->g.nx && win[2] == 0 && win[3] == ctx->g.ny;
+  auto plan2 = [ctx, probe, whole](int64_t left) {
+    return small_plan2(ctx, probe || !whole ? 1 : (int)std::min<int64_t>(left, gks::kSmallSteps));
   };
   gks::SmallPlan pl;
   gks::SmallPlan3 pl3;
@@ -759,7 +768,9 @@ gks_status gks_step_state_window(gks_ctx *ctx, const void *src, void *dst, int64
   a.V = src;
   a.Vout = dst;
   a.src_amp = source_amplitude(ctx, step);
-  GKS_CUDA(gks::launch_cart2d_step(ctx->g, a, ctx->fp64, ctx->st));
+  const gks::SmallPlan pl = may_be_small2(ctx, a) ? small_plan2(ctx, 1) : gks::SmallPlan();
+  GKS_CUDA(pl.steps > 0 ? gks::launch_cart2d_small(ctx->g, a, pl, &a.src_amp, ctx->fp64, ctx->st)
+                        : gks::launch_cart2d_step(ctx->g, a, ctx->fp64, ctx->st));
   ctx->launches += 1;
   return GKS_OK;
 }

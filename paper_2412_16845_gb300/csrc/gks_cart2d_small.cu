@@ -11,6 +11,8 @@
 //   faces   the left and lower face of every cell;
 //   update  every cell from its four faces.
 // 64^2 FP64: 4.3 us a step (general kernel 57), 100^2 FP32: 2.7 (12.4).
+// Steps over a window (the adjoint's recomputed states) take this kernel on the same grids, one step a
+// launch over the window's tiles, so that they repeat the bits of whole steps.
 // Bound: the latency of these phases (three or four barriers a step), in FP64 the FP64 pipe.  The
 // launch rule (plan) weighs the margin's work against the launches saved.
 #include <cuda_runtime.h>
@@ -47,6 +49,7 @@ struct SmallArgs {
   AxisK<T> X, Y;
   int *flag;
   int tw, th, steps, tiles_x;         // tile, steps of this launch, tiles along x
+  int wx0, wx1, wy0, wy1;             // cells to advance (a window smaller than the grid: one step only)
 };
 
 __device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
@@ -84,7 +87,8 @@ __global__ void __launch_bounds__(NT<T>) cart2d_small_kernel(const __grid_consta
   T *lx = sm + 7 * N, *hx = sm + 10 * N;              // x: sides toward the low / high face (P, QE, QH)
   T *ly = sm + 13 * N, *hy = sm + 16 * N;             // y
   T *gx = sm + 19 * N, *gy = sm + 21 * N;             // left face: GE, GH; lower face: GE (GH over ly)
-  const int X0 = (blockIdx.x % p.tiles_x) * p.tw - 2 * S, Y0 = (blockIdx.x / p.tiles_x) * p.th - 2 * S;
+  const int X0 = p.wx0 + (blockIdx.x % p.tiles_x) * p.tw - 2 * S;
+  const int Y0 = p.wy0 + (blockIdx.x / p.tiles_x) * p.th - 2 * S;
   const bool nxl = !p.perx && !p.pec[0], nxh = !p.perx && !p.pec[1];
   const bool nyl = !p.pery && !p.pec[2], nyh = !p.pery && !p.pec[3];
   const int tid = threadIdx.x;
@@ -189,7 +193,7 @@ __global__ void __launch_bounds__(NT<T>) cart2d_small_kernel(const __grid_consta
   }
   bool bad = false;
   each(2 * S, 0, [&](int i, int x, int y) {
-    if (x >= p.nx || y >= p.ny) return;
+    if (x >= p.wx1 || y >= p.wy1) return;
     const int64_t o = (int64_t)y * p.pitch + x;
     p.Vout[o] = fe[i];
     p.Vout[p.cstride + o] = fa[i];
@@ -254,8 +258,9 @@ cudaError_t launch_t(const CartGeom &g, const CartStepArgs &a, const SmallPlan &
   p.Y = make_axis<T>(a.C, a.c, g.h[1], g.h[0], -1.0);
   p.flag = a.flag;
   p.tw = pl.tw; p.th = pl.th; p.steps = pl.steps;
-  p.tiles_x = (g.nx + pl.tw - 1) / pl.tw;
-  const int grid = p.tiles_x * ((g.ny + pl.th - 1) / pl.th);
+  p.wx0 = a.window[0]; p.wx1 = a.window[1]; p.wy0 = a.window[2]; p.wy1 = a.window[3];
+  p.tiles_x = (p.wx1 - p.wx0 + pl.tw - 1) / pl.tw;
+  const int grid = p.tiles_x * ((p.wy1 - p.wy0 + pl.th - 1) / pl.th);
   constexpr int smem = N * NF * (int)sizeof(T);
   auto kern = a.limiter ? cart2d_small_kernel<T, true> : cart2d_small_kernel<T, false>;
   static SharedLimit limit;

@@ -164,6 +164,7 @@ struct SmallPlan {
   int tw = 0, th = 0, steps = 0;
   double us = 1e300;                  // estimated time per step
 };
+// (whether a grid is small does not depend on `most`: the largest tile passes the rule with one step)
 SmallPlan cart2d_small_plan(const CartGeom &g, bool fp64, int most);
 cudaError_t launch_cart2d_small(const CartGeom &g, const CartStepArgs &a, const SmallPlan &pl,
                                 const double *amp, bool fp64, cudaStream_t st);

@@ -42,7 +42,7 @@ def test_buffers_live_on_the_problems_stream(fake_torch, own):
 def test_a_wait_that_ran_out_in_backward_is_an_error(fake, fake_torch, kernel):
     """The lambda march and the recomputed steps have bounded waits; a wrong gradient is not returned."""
     from paper_2412_16845_gb300 import gks
-    p = _problem(_workload())
+    p = _problem(_workload(nx=400, ny=300))           # (smaller grids recompute without waits)
     p.forward(p.base_eps[p.design])
     fake.give_up(kernel)
     with pytest.raises(gks.GksError) as e:

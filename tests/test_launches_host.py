@@ -75,16 +75,16 @@ def _states(w, precision, *offsets):
 ])
 def test_a_callers_state_goes_to_a_kernel_that_takes_its_alignment(fake, precision, kappa, bc, src, dst, kernel):
     from paper_2412_16845_gb300 import gks
-    w = _grid((40, 30), bc)
+    w = _grid((4000, 3), bc)                          # too wide for the kernel of small grids
     keep, (p, q) = _states(w, precision, src, dst)
     s = GKSSolver.from_workload(w, precision=precision, kappa=kappa)
     fake.launched()
     if kernel is None:
         with pytest.raises(gks.GksError):
-            gks.gks_step_state_window(s.ctx, p, q, 0, 0, 40, 0, 30)
+            gks.gks_step_state_window(s.ctx, p, q, 0, 0, 40, 0, 3)
         assert not fake.launched()
     else:
-        gks.gks_step_state_window(s.ctx, p, q, 0, 0, 40, 0, 30)
+        gks.gks_step_state_window(s.ctx, p, q, 0, 0, 40, 0, 3)
         assert [kernel + "I" in k or kernel + "E" in k for k in fake.launched()] == [True]
     s.close()
 
@@ -136,3 +136,30 @@ def test_a_failed_change_of_materials_keeps_extreme_permittivities_off_the_fast_
     s.step(1)
     assert "cart2d_small_kernel" in fake.launched()[0]
     s.close()
+
+
+@pytest.mark.parametrize("precision", ["fp32", "fp64"])
+@pytest.mark.parametrize("n", [(1, 1), (5, 3), (64, 64), (100, 100), (173, 211), (288, 300), (290, 280), (24, 3600),
+                               (24, 3700), (320, 280), (500, 300), (4000, 2)])
+def test_every_step_of_a_2d_grid_takes_the_same_arithmetic(fake, n, precision):
+    """Whole steps, in any number at a time and with a probe, windowed steps and steps between a caller's
+    states: either all take the kernel of small grids or all the march."""
+    from paper_2412_16845_gb300 import gks
+    w = _grid(n, "nnpp" if n[1] > 1 else "nnnn")
+    s = GKSSolver.from_workload(w, precision=precision)
+    keep, (p, q) = _states(w, precision, 0, 0)
+    fake.launched()
+    for k in (1, 2, 3, 8, 11):
+        s.step(k)
+    x1, y1 = (n[0] + 1) // 2, (n[1] + 1) // 2
+    gks.gks_step_window(s.ctx, 3, 0, n[0], 0, n[1])
+    gks.gks_step_window(s.ctx, 2, 0, x1, 0, y1)
+    gks.gks_step_state_window(s.ctx, p, q, 0, 0, x1, 0, y1)
+    names = fake.launched()
+    gks.gks_set_objective(s.ctx, [0], [0])
+    s.step(5)
+    names += [k for k in fake.launched() if "objective" not in k]
+    s.close()
+    small = sum("cart2d_small_kernel" in k for k in names)
+    assert small in (0, len(names)), names
+    assert (small > 0) == (-(-n[0] // 24) * -(-n[1] // 24) <= 152), n      # one 24 x 24 tile per SM at most
