@@ -115,6 +115,9 @@ class _Tensor:
     def record_stream(self, s):
         self.streams.append(s.name)
 
+    def __rmul__(self, other):
+        return other * self.t
+
     def __getattr__(self, name):
         return getattr(self.t, name)
 

@@ -51,6 +51,23 @@ def test_a_wait_that_ran_out_in_backward_is_an_error(fake, fake_torch, kernel):
     p.close()
 
 
+@pytest.mark.parametrize("late", [False, True])
+def test_autograd_reports_a_wait_that_ran_out(fake, fake_torch, late):
+    from paper_2412_16845_gb300 import adjoint, gks
+    p = _problem(_workload(nx=400, ny=300))
+    e = fake_torch.tensor(p.base_eps[p.design], requires_grad=True)
+    J = adjoint._autograd_class().apply(e, p)
+    if not late:
+        J.backward()
+        assert e.grad.shape == e.shape
+    else:
+        fake.give_up(b"adjoint_tau0_kernel")
+        with pytest.raises(gks.GksError) as err:
+            J.backward()
+        assert err.value.status == gks.GKS_E_TIMEOUT
+    p.close()
+
+
 @pytest.mark.parametrize("bc", [("nrbc",) * 4, ("periodic",) * 4])
 def test_an_empty_probe_has_a_zero_gradient(fake, fake_torch, bc):
     """gks_set_objective takes an empty probe: J = 0, and no lambda acts anywhere."""
