@@ -680,7 +680,7 @@ gks_status step_impl(gks_ctx *ctx, int64_t n_steps, const int win[4], bool objec
   if (small2 && n_steps > 0) pl = plan2(n_steps);
   if (small3) {
     if (!ctx->have3) {
-      ctx->plan3 = gks::cart3d_small_plan(ctx->g, ctx->fp64);
+      ctx->plan3 = gks::cart3d_small_plan(ctx->g, a, ctx->fp64);
       ctx->have3 = true;
     }
     pl3 = ctx->plan3;

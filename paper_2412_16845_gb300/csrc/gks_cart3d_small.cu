@@ -251,12 +251,18 @@ cudaError_t launch_t(const CartGeom &g, const CartStepArgs &a, cudaStream_t st) 
 
 }  // namespace
 
-// The tile with the least estimated time, against the marching kernels' (fits to measured steps of 12^3
-// to 64 x 56 x 40 cells; FP32 tile 8 x 4 x 4: 3.9 us with one per SM, 6.6 with three, 14.6 with eight;
-// FP64 8 x 8 x 4: 23.9, 45.8 with two, 92.8 with four; marching FP32 9.2 us at 32^3, 11.3 at 48^3,
-// FP64 73.7 and 106.6).
-SmallPlan3 cart3d_small_plan(const CartGeom &g, bool fp64) {
+// The tile with the least estimated time, against the kernel that the step would take otherwise: fits to
+// steps of 24 grids of 8^3 to 120^3 cells with every tile, open sides, with and without the limiter.  A tile
+// costs its sides' work; a second FP32 tile on an SM hides the first one's latency unless shared memory holds
+// only one (8 x 8 x 8).  us a step with one, two, four and eight tiles on the busiest SM: FP32 8 x 4 x 4 4.4,
+// 6.9, 8.9, 14.9; 8 x 8 x 8 7.6, 13.9, 26.0, 49.8; FP64 8 x 8 x 4 24.5, 46.3, 93.4, 181; estimates within 10%
+// (FP32 8%, 8 x 4 x 4 alone -4%).  Otherwise: FP32 with open or periodic sides the march (8.1 at 32^3, 10.2 at
+// 48^3: crossing near 100,000 cells); with the limiter or walls the general kernel (18.8 and 22.9; limited small
+// tiles 5.8 and 11.7; crossing near 500,000); FP64 the march (48^3 107, small tiles 70; 130 x 118 x 97 929,
+// small tiles 985).
+SmallPlan3 cart3d_small_plan(const CartGeom &g, const CartStepArgs &a, bool fp64) {
   SmallPlan3 best;
+  const bool lim = a.limiter != 0;
   static int sms = 0;
   if (!sms) {
     int dev = 0, n = 0;
@@ -272,15 +278,19 @@ SmallPlan3 cart3d_small_plan(const CartGeom &g, bool fp64) {
     const int64_t ctas = (int64_t)((g.nx + b[0] - 1) / b[0]) * ((g.ny + b[1] - 1) / b[1]) *
                          ((g.nz + b[2] - 1) / b[2]);
     const double per = (double)((ctas + sms - 1) / sms);
-    const double us = fp64 ? 3.3 + per * sides[i] * 0.0217 : 2.4 + per * sides[i] * 0.00275;
+    const double us = fp64 ? 3.5 + per * sides[i] * (lim ? 0.0495 : 0.0228)
+                           : 2.5 + per * (0.3 + sides[i] * (lim ? 0.0029 : 0.0026)) +
+                                 (i == 0 ? 0.9 * (per - 1.0) : 0.0);
     if (us < best.us) {
       best.us = us;
       best.tile = i;
     }
   }
   const double kcells = 1e-3 * g.nx * g.ny * g.nz;
-  const double march = fp64 ? 28.0 + 0.62 * kcells : 8.5 + 0.015 * kcells;
-  if (!(best.us < march)) best.tile = -1;
+  const double other = fp64                               ? cart3d_tau0_f64_us(g, lim)
+                       : cart3d_side_supported(g, a, fp64) ? 8.5 + 0.015 * kcells
+                                                           : 15.0 + (lim ? 0.075 : 0.06) * kcells;
+  if (!(best.us < other)) best.tile = -1;
   return best;
 }
 

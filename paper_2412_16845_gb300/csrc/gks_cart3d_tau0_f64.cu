@@ -280,17 +280,7 @@ __global__ void __launch_bounds__(WARPS * 32, 2) cart3d_tau0_f64_kernel(const __
   if (__any_sync(FULL, bad) && lane == 0) atomicOr(p.flag, 1);
 }
 
-}  // namespace
-
-bool cart3d_tau0_f64_supported(const CartStepArgs &a) {
-  return !a.mu && a.eps_normal && a.C[1] == 0.0 && a.C[3] == 0.0 && a.C[4] == 0.0 && a.C[0] > 0.0;
-}
-
-cudaError_t launch_cart3d_tau0_f64(const CartGeom &g, const CartStepArgs &a, cudaStream_t st) {
-  static SharedLimit limit;
-  const cudaError_t e = limit.raise(WARPS * MAXR * NST * 32 * 8, cart3d_tau0_f64_kernel<false>,
-                                    cart3d_tau0_f64_kernel<true>);
-  if (e != cudaSuccess) return e;
+int sm_count() {
   static int sms = 0;
   if (!sms) {
     int dev = 0, n = 0;
@@ -298,16 +288,22 @@ cudaError_t launch_cart3d_tau0_f64(const CartGeom &g, const CartStepArgs &a, cud
     cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
     sms = n > 0 ? n : 1;
   }
-  Args p;
+  return sms;
+}
+
+// Lane axis, rows per warp and planes per chunk: the least FP64 work on the busiest scheduler for
+// one to four warps on each.  A chunk costs about 0.48 of a row (plane) more; one warp alone on a
+// scheduler does not hide its loads (an eighth); strided access along the lanes costs a few
+// percent.
+struct Plan {
+  int axis = 0, strips = 0, nrow = 0, nmarch = 0, R = 0, Z = 0;
+};
+
+Plan plan_march(const CartGeom &g) {
   const int n[3] = {g.nx, g.ny, g.nz};
-  const int64_t stride[3] = {1, g.pitch, g.plane};
-  // Lane axis, rows per warp and planes per chunk: the least FP64 work on the busiest scheduler for
-  // one to four warps on each.  A chunk costs about 0.48 of a row (plane) more; one warp alone on a
-  // scheduler does not hide its loads (an eighth); strided access along the lanes costs a few
-  // percent.
-  const int64_t sched = (int64_t)sms * WARPS;
+  const int64_t sched = (int64_t)sm_count() * WARPS;
   double best = 1e300;
-  int lane_axis = 0;
+  Plan pl;
   for (int ax = 0; ax < 3; ++ax) {
     const int nl = n[ax], nr = n[(ax + 1) % 3], nm = n[(ax + 2) % 3];
     const int strips = (nl + WL - 1) / WL;
@@ -321,12 +317,42 @@ cudaError_t launch_cart3d_tau0_f64(const CartGeom &g, const CartStepArgs &a, cud
                             (nw > sched ? 1.0 : 1.125) * (ax == 0 ? 1.0 : 1.25);
         if (cost < best * 0.999) {
           best = cost;
-          lane_axis = ax;
-          p.strips = strips; p.nrow = nrow; p.nmarch = nmarch; p.R = R; p.Z = Z;
+          pl.axis = ax; pl.strips = strips; pl.nrow = nrow; pl.nmarch = nmarch; pl.R = R; pl.Z = Z;
         }
       }
     }
   }
+  return pl;
+}
+
+}  // namespace
+
+// Fits to steps of 24 grids of 32^3 to 120^3 cells, within 10%: a row of a plane takes two warps of a
+// scheduler 16.7 us together, a single one 12.1 (loads not hidden); lanes along y or z take 13% more.
+double cart3d_tau0_f64_us(const CartGeom &g, bool limited) {
+  const Plan pl = plan_march(g);
+  const int64_t sched = (int64_t)sm_count() * WARPS;
+  const int64_t waves = ((int64_t)pl.strips * pl.nrow * pl.nmarch + sched - 1) / sched;
+  const double two = limited ? 30.5 : 16.7, one = limited ? 21.6 : 12.1;
+  return (pl.R + 0.48) * (pl.Z + 0.48) * ((double)(waves / 2) * two + (double)(waves % 2) * one) *
+         (pl.axis == 0 ? 1.0 : 1.13);
+}
+
+bool cart3d_tau0_f64_supported(const CartStepArgs &a) {
+  return !a.mu && a.eps_normal && a.C[1] == 0.0 && a.C[3] == 0.0 && a.C[4] == 0.0 && a.C[0] > 0.0;
+}
+
+cudaError_t launch_cart3d_tau0_f64(const CartGeom &g, const CartStepArgs &a, cudaStream_t st) {
+  static SharedLimit limit;
+  const cudaError_t e = limit.raise(WARPS * MAXR * NST * 32 * 8, cart3d_tau0_f64_kernel<false>,
+                                    cart3d_tau0_f64_kernel<true>);
+  if (e != cudaSuccess) return e;
+  Args p;
+  const int n[3] = {g.nx, g.ny, g.nz};
+  const int64_t stride[3] = {1, g.pitch, g.plane};
+  const Plan pl = plan_march(g);
+  const int lane_axis = pl.axis;
+  p.strips = pl.strips; p.nrow = pl.nrow; p.nmarch = pl.nmarch; p.R = pl.R; p.Z = pl.Z;
   double h[3];
   for (int r = 0; r < 3; ++r) {
     const int ax = (lane_axis + r) % 3;

@@ -174,7 +174,7 @@ struct SmallPlan3 {
   int tile = -1;
   double us = 1e300;                  // estimated time per step
 };
-SmallPlan3 cart3d_small_plan(const CartGeom &g, bool fp64);
+SmallPlan3 cart3d_small_plan(const CartGeom &g, const CartStepArgs &a, bool fp64);
 cudaError_t launch_cart3d_small(const CartGeom &g, const CartStepArgs &a, const SmallPlan3 &pl,
                                 bool fp64, cudaStream_t st);
 // FP32 3-D step with tau = 0 where the side-split kernel would run (gks_cart3d_tau0.cu).
@@ -182,6 +182,7 @@ bool cart3d_tau0_supported(const CartGeom &g, const CartStepArgs &a);
 cudaError_t launch_cart3d_tau0(const CartGeom &g, const CartStepArgs &a, cudaStream_t st);
 // FP64 3-D step with tau = 0 and mu = 1 (gks_cart3d_tau0_f64.cu).
 bool cart3d_tau0_f64_supported(const CartStepArgs &a);
+double cart3d_tau0_f64_us(const CartGeom &g, bool limited);   // its estimated step
 cudaError_t launch_cart3d_tau0_f64(const CartGeom &g, const CartStepArgs &a, cudaStream_t st);
 // 2-D TM step with divergence cleaning (state Ez, Hx, Hy, psi; mu = 1).
 // Divergence-cleaning system on a 3-D grid: V = (E, H, phi, psi), 8 components.

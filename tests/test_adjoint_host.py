@@ -78,3 +78,113 @@ def test_an_empty_probe_has_a_zero_gradient(fake, fake_torch, bc):
     g = p.backward()
     assert J == 0.0 and g.t.shape == (p.design.size,) and not g.t.any()
     p.close()
+
+
+def _context(precision="fp32", n=(40, 30), **kw):
+    from paper_2412_16845_gb300 import gks
+    s = gks.GKSSolver(gks.SolverSpec(dim=len(n), n=n, lo=(0.0,) * len(n), hi=(1.0,) * len(n),
+                                     bc=kw.pop("bc", ("nrbc",) * (2 * len(n))), cfl=0.3, precision=precision, **kw))
+    _, nbytes = gks.gks_state_layout(s.ctx)
+    bufs = [np.zeros(nbytes + 32, dtype=np.uint8) for _ in range(4)]
+    return s, bufs, [(b.ctypes.data + 15) // 16 * 16 for b in bufs]
+
+
+BAD_WINDOWS = [(-1, 4, 0, 4), (0, 41, 0, 4), (0, 4, -1, 4), (0, 4, 0, 31), (5, 5, 0, 4), (6, 5, 0, 4), (0, 4, 7, 7)]
+
+
+@pytest.mark.parametrize("window", BAD_WINDOWS)
+def test_windows_outside_the_grid_are_refused(fake, window):
+    from paper_2412_16845_gb300 import gks
+    s, keep, (a, b, c, d) = _context()
+    gks.gks_set_objective(s.ctx, [3], [4])
+    with pytest.raises(gks.GksError) as e:
+        gks.gks_step_state_window(s.ctx, a, b, 0, *window)
+    assert e.value.status == gks.GKS_E_ARG
+    with pytest.raises(gks.GksError) as e:
+        gks.gks_adjoint_step_window(s.ctx, a, b, c, d, a, True, *window)
+    assert e.value.status == gks.GKS_E_ARG
+    assert not fake.launched()[1:]                     # (the fill of eps at creation)
+    s.close()
+
+
+def test_arguments_of_the_window_calls(fake):
+    from paper_2412_16845_gb300 import gks
+    s, keep, (a, b, c, d) = _context()
+    gks.gks_set_objective(s.ctx, [3], [4])
+    win = (0, 40, 0, 30)
+    for src, dst, step in ((None, b, 0), (a, None, 0), (a, a, 0), (a, b, -1), (a + 2, b, 0), (a, b + 1, 0)):
+        with pytest.raises(gks.GksError) as e:
+            gks.gks_step_state_window(s.ctx, src, dst, step, *win)
+        assert e.value.status == gks.GKS_E_ARG
+    for vn, vn1, lin, lout, g in ((None, b, c, d, a), (a, None, c, d, a), (a, b, None, d, a), (a, b, c, None, a),
+                                  (a, b, c, c, a), (a, b, c, d, None), (a, b, c + 2, d, a)):
+        with pytest.raises(gks.GksError) as e:
+            gks.gks_adjoint_step_window(s.ctx, vn, vn1, lin, lout, g, True, *win)
+        assert e.value.status == gks.GKS_E_ARG
+    s.close()
+    # what the whole-grid calls refuse
+    for kw, step_too in (({"n": (8, 8, 8)}, True), ({"phm": (0.0, 1.0)}, True), ({"limiter": "vanleer"}, False),
+                         ({"bc": ("pec", "pec", "nrbc", "nrbc")}, False)):
+        s, keep, (a, b, c, d) = _context(**kw)
+        with pytest.raises(gks.GksError) as e:
+            gks.gks_adjoint_step_window(s.ctx, a, b, c, d, a, False, 0, 4, 0, 4)
+        assert e.value.status == gks.GKS_E_UNSUPPORTED
+        if step_too:
+            with pytest.raises(gks.GksError) as e:
+                gks.gks_step_state_window(s.ctx, a, b, 0, 0, 4, 0, 4)
+            assert e.value.status == gks.GKS_E_UNSUPPORTED
+        s.close()
+
+
+def _brute_lambda(p, w):
+    """Cells where lambda^n is not zero and acts on the gradient, by dilating masks two cells a step."""
+    nx, ny = w.n
+    per = (w.bc[0] == "periodic", w.bc[2] == "periodic")
+
+    def grow(m):
+        for axis, wrap in ((1, per[0]), (0, per[1])):
+            acc = m.copy()
+            for k in (1, 2):
+                for sgn in (1, -1):
+                    r = np.roll(m, sgn * k, axis=axis)
+                    if not wrap:
+                        idx = [slice(None)] * 2
+                        idx[axis] = slice(0, k) if sgn > 0 else slice(-k, None)
+                        r[tuple(idx)] = False
+                    acc |= r
+            m = acc
+        return m
+    lam, act = [None] * (p.N + 1), [None] * (p.N + 1)
+    m = np.zeros((ny, nx), bool)
+    m.ravel()[w.probe] = True
+    for n in range(p.N, -1, -1):
+        lam[n] = m
+        m = grow(m)
+    # lambda^n acts on the gradient through lambda^k, k <= n, beside a design cell (k's step reads two cells)
+    a = np.zeros((ny, nx), bool)
+    a.ravel()[w.design] = True
+    for n in range(0, p.N + 1):
+        a = grow(a) if n else a
+        act[n] = a
+    return lam, act
+
+
+@pytest.mark.parametrize("bc", [("nrbc",) * 4, ("periodic",) * 4, ("periodic", "periodic", "nrbc", "nrbc")])
+@pytest.mark.parametrize("design,probe", [
+    (((8, 16), (6, 14)), ((24, 27), (15, 18))), (((1, 4), (2, 5)), ((36, 39), (28, 31))),
+    (((30, 40), (0, 3)), ((0, 2), (0, 2))), (((5, 6), (5, 6)), ((33, 34), (25, 26))),
+])
+def test_lambda_windows_hold_every_cell_that_acts(fake_torch, bc, design, probe):
+    w = _workload(bc=bc, steps=14, design=design, probe=probe)
+    p = _problem(w)
+    lam, act = _brute_lambda(p, w)
+    for n in range(p.N):
+        need = lam[n] & act[n]
+        win = p._lambda_window(n)
+        if win is None:
+            assert not need.any(), n
+            continue
+        x0, x1, y0, y1 = win
+        need[y0:y1, x0:x1] = False
+        assert not need.any(), (n, win)
+    p.close()

@@ -24,11 +24,19 @@ MARCH_2D = [((61, 1300), "nnnn", None), ((62, 1300), "nnpp", None), ((63, 1301),
 
 # 3-D, FP64: strips of 30 cells, up to 8 rows and any number of planes per warp; FP32: tiles of 64 columns x
 # 10 rows, chunks of planes (open and periodic sides)
-MARCH_3D = [((33, 9, 600), "nnmmpp", None, "fp64"), ((30, 17, 330), "mmmmnn", None, "fp64"),
-            ((91, 10, 200), "ppnnmn", None, "fp64"), ((33, 9, 601), "nnnnnn", "vanleer", "fp64"),
-            ((59, 2, 1400), "mmnnpp", None, "fp64"), ((9, 400, 60), "nnmmnn", None, "fp64"),
+MARCH_3D = [((33, 9, 600), "nnmmpp", None, "fp64"), ((60, 17, 170), "mmmmnn", None, "fp64"),
+            ((90, 17, 120), "nnmmpp", None, "fp64"), ((60, 9, 310), "ppnnmn", None, "fp64"),
+            ((33, 9, 601), "nnnnnn", "vanleer", "fp64"), ((59, 2, 1400), "mmnnpp", None, "fp64"),
+            ((9, 400, 60), "nnmmnn", None, "fp64"), ((600, 33, 9), "mmnnpp", None, "fp64"),
+            ((97, 89, 91), "nnmmnn", None, "fp64"),        # chunks of 4 rows x 7 planes
             ((65, 51, 50), "nnppnn", None, "fp32"), ((129, 41, 31), "ppnnpp", None, "fp32"),
             ((63, 1, 2600), "nnppnn", None, "fp32"), ((64, 30, 90), "nnnnnn", None, "fp32")]
+
+# 3-D grids of several tiles per SM that take one tile per CTA all the same: FP64, and FP32 where the march
+# does not run (limiter, walls)
+TILES_3D = [((57, 43, 66), "nnnnnn", "vanleer", "fp32"), ((48, 50, 47), "mmnmpp", None, "fp32"),
+            ((61, 40, 33), "nmppmm", "vanleer", "fp32"), ((63, 41, 30), "nnmmpp", None, "fp64"),
+            ((45, 34, 27), "nnpppp", None, "fp32")]
 
 
 @pytest.fixture(scope="module", autouse=True)
@@ -66,6 +74,6 @@ def test_2d(n, bc, limiter, precision):
     _check(grid(n, bc, limiter), precision, 5)
 
 
-@pytest.mark.parametrize("n,bc,limiter,precision", MARCH_3D)
+@pytest.mark.parametrize("n,bc,limiter,precision", MARCH_3D + TILES_3D)
 def test_3d(n, bc, limiter, precision):
     _check(grid(n, bc, limiter), precision, 2)

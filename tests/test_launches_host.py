@@ -163,3 +163,55 @@ def test_every_step_of_a_2d_grid_takes_the_same_arithmetic(fake, n, precision):
     small = sum("cart2d_small_kernel" in k for k in names)
     assert small in (0, len(names)), names
     assert (small > 0) == (-(-n[0] // 24) * -(-n[1] // 24) <= 152), n      # one 24 x 24 tile per SM at most
+
+
+def _kernel_of(fake, n, bc, limiter, precision, kappa=0.0):
+    s = GKSSolver.from_workload(_grid(n, bc, limiter), precision=precision, kappa=kappa)
+    fake.launched()
+    s.step(1)
+    names = fake.launched()
+    s.close()
+    return names[0]
+
+
+# what was timed (us a step): the faster one of one tile per CTA and of the kernel the step takes otherwise
+@pytest.mark.parametrize("n,bc,limiter,precision,small", [
+    ((64, 64, 64), "nnnnnn", None, "fp64", True),           # 162, march 261
+    ((80, 80, 80), "nnnnnn", None, "fp64", True),           # 321, 331
+    ((90, 80, 70), "nnnnnn", None, "fp64", False),          # 342, 308
+    ((130, 118, 97), "nnnnnn", None, "fp64", False),        # 985, 929
+    ((33, 9, 600), "nnnnnn", None, "fp64", False),          # 175, 162
+    ((64, 64, 64), "nnnnnn", "vanleer", "fp64", True),      # 361, 493
+    ((80, 80, 80), "nnnnnn", "vanleer", "fp64", False),     # 720, 620
+    ((40, 40, 40), "nnnnnn", None, "fp32", True),           # 8.0, 9.8
+    ((56, 48, 40), "nnnnnn", None, "fp32", False),          # 10.8, 9.8
+    ((56, 48, 40), "nnnnnn", "vanleer", "fp32", True),      # 11.7, general kernel 23.0
+    ((64, 64, 64), "mmmmmm", None, "fp32", True),           # 22.1, 35.3
+    ((90, 80, 70), "mmmmmm", None, "fp32", False),          # 44.8, 43.7
+])
+def test_3d_rule_takes_the_faster_kernel(fake, n, bc, limiter, precision, small):
+    assert ("cart3d_small_kernel" in _kernel_of(fake, n, bc, limiter, precision)) == small
+
+
+def test_45_34_27_takes_the_tile_that_was_fastest(fake):
+    """8 x 4 x 4 tiles: 7.0 us a step; 4 x 4 x 4: 9.1, 8 x 8 x 4: 7.6, 8 x 8 x 8: 7.9."""
+    assert "cart3d_small_kernelIfLi2E" in _kernel_of(fake, (45, 34, 27), "nnpppp", None, "fp32")
+
+
+def test_the_parity_grids_take_the_kernels_they_are_for(fake):
+    """The grids of tests/test_gpu_tau0_march.py, test_gpu_slab_march.py and test_gpu_cart2d_general.py."""
+    from tests import test_gpu_cart2d_general as general
+    from tests import test_gpu_slab_march as slabs
+    from tests import test_gpu_tau0_march as march
+    for n, bc, limiter in march.MARCH_2D:
+        assert "cart2d_tau0_kernel" in _kernel_of(fake, n, bc, limiter, "fp32"), n
+        assert "cart2d_tau0_f64_kernel" in _kernel_of(fake, n, bc, limiter, "fp64"), n
+    for n, bc, limiter, precision in march.MARCH_3D:
+        kernel = "cart3d_tau0_f64_kernel" if precision == "fp64" else "cart3d_tau0_kernel"
+        assert kernel in _kernel_of(fake, n, bc, limiter, precision), n
+    for n, bc, limiter, precision in march.TILES_3D:
+        assert "cart3d_small_kernel" in _kernel_of(fake, n, bc, limiter, precision), n
+    for n, bc in general.STAGED:
+        assert "cart2d_step_kernel_s" in _kernel_of(fake, n, bc, None, "fp32", general.KAPPA), n
+    for _, _, _, precision, local, kernel in slabs.SLABS:
+        assert kernel in _kernel_of(fake, local, "nn" * len(local), None, precision), local
