@@ -204,11 +204,15 @@ __global__ void __launch_bounds__(BX *kBY<T>, 1)
     return !p.per[a] && ((i < 0 && !p.pec[2 * a]) || (i >= p.n[a] && !p.pec[2 * a + 1]));
   };
   const bool gx = beyond(0, x), gy = beyond(1, y);
-  // in-plane offset and mirror flags of the thread's column, and of the ring entry it stages
+  // In-plane offset and mirror flags of the thread's column, and of the ring entry it stages.  No cell of the
+  // grid reads columns past the two ghost layers; they are wrapped so that a warp's lanes copy from different
+  // addresses.  (Clamped past an open side, or to the far side's cell past a wall, they were one cell, and a
+  // warp's copies from one address go one after the other: 32^3 open 18.8 us a step, 100 x 90 x 80 70, where
+  // periodic sides took 8.4 and 42.)
   bool mx, my, rmx, rmy;
   auto column = [&](int cx, int cy, bool &ax, bool &ay) {
     return (int64_t)image8(cy, p.n[1], p.per[1], p.pec[2], p.pec[3], ay) * p.pitch +
-           image8(cx, p.n[0], p.per[0], p.pec[0], p.pec[1], ax);
+           image8(cx, p.n[0], p.per[0] || cx > p.n[0] + 1, p.pec[0], p.pec[1], ax);
   };
   const int64_t own = column(x, y, mx, my);
   const bool ringer = tid < NRING;
@@ -217,24 +221,16 @@ __global__ void __launch_bounds__(BX *kBY<T>, 1)
   else if (tid < 2 * PX) { rpy = BY + 1; rpx = tid - PX; }
   else if (ringer) { rpy = 1 + ((tid - 2 * PX) >> 1); rpx = ((tid - 2 * PX) & 1) ? PX - 1 : 0; }
   const int64_t rown = column(x0 - 2 + rpx, y0 - 2 + rpy, rmx, rmy);
-  // No cell of the grid reads columns past the two ghost layers: they are not fetched, and what their lanes
-  // compute from stale entries is not used.  (Past an open or closed x side their images are all one cell,
-  // and copies of a warp's lanes from one address go one after the other: 32^3 open 18.8 us a step, 100 x 90
-  // x 80 70, where periodic sides took 8.4 and 42.)
-  const bool on = x <= p.n[0] + 1 && y <= p.n[1] + 1;
-  const bool rim = ringer && x0 - 2 + rpx <= p.n[0] + 1 && y0 - 2 + rpy <= p.n[1] + 1;
   // Plane z into slot q by asynchronous copies: each thread its own entry and, the first NRING, one of the
   // ring; they land while the plane before is worked on.
   auto fetch = [&](int z, int q) {
     bool az;
     const int64_t o = (int64_t)image8(z, p.n[2], p.per[2], p.pec[4], p.pec[5], az) * p.plane;
     const T *g = p.V + (o + own);
-    if (on) {
 #pragma unroll
-      for (int c = 0; c < 8; ++c, g += p.cstride) copy_async(&s.V[q][c][ty + 1][tx + 1], g);
-      copy_async(&s.V[q][8][ty + 1][tx + 1], p.eps + (o + own));
-    }
-    if (rim) {
+    for (int c = 0; c < 8; ++c, g += p.cstride) copy_async(&s.V[q][c][ty + 1][tx + 1], g);
+    copy_async(&s.V[q][8][ty + 1][tx + 1], p.eps + (o + own));
+    if (ringer) {
       g = p.V + (o + rown);
 #pragma unroll
       for (int c = 0; c < 8; ++c, g += p.cstride) copy_async(&s.V[q][c][rpy][rpx], g);
@@ -258,7 +254,7 @@ __global__ void __launch_bounds__(BX *kBY<T>, 1)
     const bool az = !p.per[2] && ((z < 0 && p.pec[4]) || (z >= p.n[2] && p.pec[5]));
     if (any_x | az) {
       mirror(ty + 1, tx + 1, q, mx, my, az);
-      if (rim) mirror(rpy, rpx, q, rmx, rmy, az);
+      if (ringer) mirror(rpy, rpx, q, rmx, rmy, az);
     }
   };
   T vm[8], v0[8], vp[8], em, e0, ep;                  // planes z-1, z, z+1
