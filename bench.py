@@ -285,7 +285,8 @@ def reduced_gpu_results(stream_ptr, path):
     np.savez(path, **out)
 
 
-# The 3-D FP32 step kernel (cart3d_tau0_kernel) is bound by instruction issue: its ncu summary
+# The 3-D FP32 step kernel (cart3d_tau0_kernel) is nearest to the issue ceiling (half of it; latency at 12
+# warps an SM keeps it there): its ncu summary
 # (profiles/cart3d_tau0_maxwell3d_sphere_fp32.md) counts 426 thread-instructions per cell at
 # 160^3, where 20% of the 64-column tiles lie past the grid, i.e. about 355 per cell on a grid of
 # whole tiles such as 256^3.  The issue peak is 152 SMs x 4 schedulers x 32 threads x 2.07 GHz.

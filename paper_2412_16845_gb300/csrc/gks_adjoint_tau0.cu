@@ -474,9 +474,9 @@ cudaError_t launch_adjoint_tau0(const CartGeom &g, const AdjointArgs &a, cudaStr
     sms = n > 0 ? n : 1;
   }
   // Rows a chunk (which computes two rows more): one wave of five CTAs per SM while that takes 40 rows or
-  // fewer, past that about four waves, 24 rows or more.  2048 x 2048: one wave (25 to 28 rows) 38 us, 24
-  // (1.02 waves) 44, 14 rows 36; 1448 x 1448: one wave (12) 18.9, 8: 21.6; 2900 x 2900: one wave (47)
-  // 61.2, 24: 61.6, 16: 62.8.
+  // fewer, past that about four waves, 24 rows or more.  us a step: 1448 x 1448 one wave (12 rows) 18.8, 8:
+  // 21.5, 14: 21.1; 2048 x 2048 one wave (25) 33.9, 24 (1.02 waves) 43.7, 28: 37.7, 14: 35.8; 2900 x 2900 24
+  // rows 61.5, 16: 62.8, 48: 61.0, 32: 67.6; 4096 x 4096 24 rows 111.0, 16: 113.8, 32: 112.7.
   const int wrows = p.wy1 - p.wy0, strips = (p.wx1 - p.wx0 + W - 1) / W;
   const int nw = std::min(WARPS, strips);
   p.ntiles = (strips + nw - 1) / nw;

@@ -665,10 +665,10 @@ cudaError_t launch_f32(const CartGeom &g, const CartStepArgs &a, cudaStream_t st
   const int nw = std::min(WARPS, strips);
   p.ntiles = (strips + nw - 1) / nw;
   // Rows a chunk: one wave of six CTAs per SM while that takes 24 rows or fewer; past that about eight
-  // waves, chunks of 16 rows or more (a chunk's prologue costs about a row and a half).  At 2048 x 2048
-  // one wave of 21 or 22 rows and 8 to 14 rows take 30 to 31 us, 16 (1.3 waves) 32.4, 20 (1.02) 33.4;
-  // 1448 x 1448: one wave (10) 15.5, 8: 17.4; 2900 x 2900: 16 rows 52.2, one wave (39) 53.7;
-  // 4096 x 4096: 16 rows 90.8, 10: 93.2.
+  // waves, chunks of 16 rows or more (a chunk's prologue costs about a row and a half).  us a step (open sides,
+  // a line source): 1448 x 1448 one wave (10 rows) 16.0, 8: 18.0, 12: 18.4, 16: 23.3; 2048 x 2048 one wave (21)
+  // 35.3, 8 to 14 rows 33.0 to 35.4, 16 (1.3 waves) 37.4, 24: 38.7; 2900 x 2900 16 rows 56.4, 10: 55.4, 24:
+  // 58.0, 48: 67.8; 4096 x 4096 16 rows 99.5, 12 and 14: 99.1, 8: 102.6, 24: 103.8.
   const int64_t resident = (int64_t)sms * 6;
   const int64_t fit = std::max<int64_t>(1, resident / p.ntiles);
   int rows = std::max(2, (int)((wrows + fit - 1) / fit));

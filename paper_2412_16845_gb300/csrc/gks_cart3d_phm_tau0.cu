@@ -23,7 +23,7 @@
 // exchanges gradients and rebuilds both sides of every face, issues 1865 a cell.
 // 150 x 139 x 128 FP32: 126 us a step (general kernel: 277).  Bound: instruction issue, 72% busy with 12
 // warps an SM (41% before the copies); BY = 14 and 16 spill below 150 registers (190, 198 us), BY = 10
-// carries a larger ring (147 us).  FP64 takes BY = 8 for its 255 registers.
+// carries a larger ring (147 us).  FP64 takes BY = 8 for its 255 registers, and spills 304 bytes all the same.
 #include <cuda_runtime.h>
 
 #include <type_traits>

@@ -8,8 +8,10 @@
 // With tau = 0 a cell sends 6 values to a neighbour instead of 12 and a face carries 4 components
 // instead of 6: 81 paired instructions a cell pair's worth of flux and update instead of 220, half the
 // shuffles and shared-memory exchange, and the z-sides fit in registers (no tensor memory).
-// Bound: instruction issue, then the two CTA barriers a plane.  256^3: 334 us a step, the side-split
-// kernel 525; 14 row warps 348, two CTAs of 6 row warps 360.
+// Bound: latency at 12 warps an SM.  Issue slots are 49.5% active at 160^3; the stalls per issue are
+// dependencies 1.5, shared memory 1.0 and the two CTA barriers a plane 0.8.  256^3: 310 to 334 us a step (back
+// to back; with a state copied before and after ten steps), the side-split kernel 525; 14 row warps 348, two CTAs
+// of 6 row warps 360.
 #include <cuda_runtime.h>
 
 #include "gks_internal.h"
@@ -612,8 +614,9 @@ cudaError_t launch_cart3d_tau0(const CartGeom &g, const CartStepArgs &a, cudaStr
   }
   // z chunks: one CTA per SM; pick the chunk count that fills whole waves best.  A CTA's fixed
   // cost -- staging its first four planes with nothing to overlap them, the z-vectors of the
-  // plane below its chunk and the closing z-face -- counts as 2.7 planes of work: the value that
-  // fits measured step times at 256^3 over 1 to 32 chunks (7 chunks, 0.511 ms; 16, 0.529 ms)
+  // plane below its chunk and the closing z-face -- counts as 2.7 planes of work.  The rule takes the fastest
+  // count of 1 to 32 at four sizes (us a step): 256^3 7 chunks 310, 4: 317, 16: 326, 1: 410; 160^3 3: 106,
+  // 5: 120; 200 x 128 x 90 5: 72, 2: 88; 300 x 200 x 100 3: 143, 5: 154.
   constexpr double kChunkCost = 2.7;
   const int64_t tiles = (int64_t)gx * gy;
   int zchunks = 1;

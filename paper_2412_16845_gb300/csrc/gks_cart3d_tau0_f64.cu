@@ -1,11 +1,13 @@
 // 3-D GKS step in FP64 for tau = 0 and mu = 1 (the pair flux of gks_pair3.cuh), van Leer slopes
 // optional; any boundary kind.
 //
-// Bound: the FP64 pipe.  A GB300 issues one FP64 warp instruction per 64 cycles and scheduler
-// (measured; one warp with independent instructions fills it), so the time is the number of FP64
-// operations (162 and four reciprocals a cell; the general kernel runs 763) times how unevenly they
-// are spread over the 608 schedulers.  Everything else -- loads, shuffles, shared memory, index
-// arithmetic, uncoalesced access -- has 64 issue slots per FP64 instruction and is free.
+// Bound: the FP64 pipe, then latency.  A GB300 issues one FP64 warp instruction per 64 cycles and
+// scheduler (measured; one warp with independent instructions fills it), so the least time is the number of
+// FP64 operations (162 and four reciprocals a cell; the general kernel runs 763) times how unevenly they are
+// spread over the 608 schedulers.  The pipe is 79% busy at 120^3 (the 2-D FP64 march, which loads two rows
+// ahead, 83%): a pass uses its loads and shuffles where it issues them, and two warps a scheduler do not hide
+// all of it (stalls per issue: wait 7.2, short scoreboard 6.7, long scoreboard 3.9).  Issue slots themselves
+// -- index arithmetic, uncoalesced access -- are plenty, 64 per FP64 instruction.
 //
 // Layout.  Warps are independent.  One warp takes a strip of 30 cells along the lane axis, up to 8
 // rows of the row axis and a chunk of planes of the march axis.  It walks the rows of a plane in
@@ -14,7 +16,8 @@
 // along the lane axis come from shuffles.  Work computed twice: 2 of 32 lanes, and about a third of
 // a row (plane) per chunk of rows (planes).  The three roles may be any cyclic renaming of x, y, z
 // (the flux is the same under it), so the lane axis is the one whose length fills strips best.
-// 130 x 118 x 97: 0.99 ms a step, the general kernel 2.59; the arithmetic alone 0.46.
+// 130 x 118 x 97: 0.93 ms a step, the general kernel 2.59; the arithmetic alone 0.46, with the halo cells
+// and the uneven last wave of this split 0.67.
 #include <cuda_runtime.h>
 
 #include <algorithm>
