@@ -656,12 +656,13 @@ bool may_be_small2(const gks_ctx *ctx, const gks::CartStepArgs &a) {
          gks::cart2d_tau0_supported(ctx->g, a, ctx->fp64);
 }
 
-gks::SmallPlan small_plan2(gks_ctx *ctx, int most) {
+gks::SmallPlan small_plan2(gks_ctx *ctx, int most, const int win[4]) {
   if (!ctx->have2[most]) {
     ctx->plan2[most] = gks::cart2d_small_plan(ctx->g, ctx->fp64, most);
     ctx->have2[most] = true;
   }
-  return ctx->plan2[most];
+  return most == 1 && ctx->plan2[1].steps > 0 ? gks::cart2d_small_step_plan(win, ctx->fp64)
+                                              : ctx->plan2[most];
 }
 
 // Advance n_steps over the window [x0, x1) x [y0, y1) (2-D) or the whole mesh.
@@ -672,8 +673,9 @@ gks_status step_impl(gks_ctx *ctx, int64_t n_steps, const int win[4], bool objec
                       gks::cart3d_tau0_f64_supported(a);
   const bool probe = objective && ctx->np > 0;       // needs the state after every step
   const bool whole = win[0] == 0 && win[1] == ctx->g.nx && win[2] == 0 && win[3] == ctx->g.ny;
-  auto plan2 = [ctx, probe, whole](int64_t left) {
-    return small_plan2(ctx, probe || !whole ? 1 : (int)std::min<int64_t>(left, gks::kSmallSteps));
+  auto plan2 = [ctx, probe, whole, win](int64_t left) {
+    const int most = probe || !whole ? 1 : (int)std::min<int64_t>(left, gks::kSmallSteps);
+    return small_plan2(ctx, most, win);
   };
   gks::SmallPlan pl;
   gks::SmallPlan3 pl3;
@@ -768,7 +770,7 @@ gks_status gks_step_state_window(gks_ctx *ctx, const void *src, void *dst, int64
   a.V = src;
   a.Vout = dst;
   a.src_amp = source_amplitude(ctx, step);
-  const gks::SmallPlan pl = may_be_small2(ctx, a) ? small_plan2(ctx, 1) : gks::SmallPlan();
+  const gks::SmallPlan pl = may_be_small2(ctx, a) ? small_plan2(ctx, 1, win) : gks::SmallPlan();
   GKS_CUDA(pl.steps > 0 ? gks::launch_cart2d_small(ctx->g, a, pl, &a.src_amp, ctx->fp64, ctx->st)
                         : gks::launch_cart2d_step(ctx->g, a, ctx->fp64, ctx->st));
   ctx->launches += 1;

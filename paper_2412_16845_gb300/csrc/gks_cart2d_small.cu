@@ -215,8 +215,8 @@ int sm_count() {
 }
 
 // Tile and steps per launch with the least estimated time per step: a launch with its loads, the
-// phases' latency per step, and the work of the shrinking region on one SM.
-SmallPlan plan(const CartGeom &g, bool fp64, int most) {
+// phases' latency per step, and the work of the shrinking region on one SM; at most per_sm CTAs an SM.
+SmallPlan plan(int nx, int ny, bool fp64, int most, int per_sm = 1) {
   const double launch = 2.2, phase = fp64 ? 1.2 : 1.0, cell = fp64 ? 0.0120 : 0.0020;   // us
   const int sms = sm_count();
   SmallPlan best;
@@ -224,8 +224,8 @@ SmallPlan plan(const CartGeom &g, bool fp64, int most) {
   for (int tw : sizes)
     for (int th : sizes) {
       if (th > tw || tw > 3 * th) continue;
-      const int64_t ctas = (int64_t)((g.nx + tw - 1) / tw) * ((g.ny + th - 1) / th);
-      if (ctas > sms) continue;
+      const int64_t ctas = (int64_t)((nx + tw - 1) / tw) * ((ny + th - 1) / th);
+      if (ctas > (int64_t)sms * per_sm) continue;
       double work = 0.0;
       for (int S = 1; S <= std::min(most, kMaxSteps); ++S) {
         if (tw + 4 * S > PW || th + 4 * S > PW) break;
@@ -272,10 +272,18 @@ cudaError_t launch_t(const CartGeom &g, const CartStepArgs &a, const SmallPlan &
 }  // namespace
 
 SmallPlan cart2d_small_plan(const CartGeom &g, bool fp64, int most) {
-  SmallPlan pl = plan(g, fp64, most);
+  SmallPlan pl = plan(g.nx, g.ny, fp64, most);
   const double march = fp64 ? 12.0 : 6.0;             // the marching kernels' step on such a grid
   if (!(pl.us < march)) pl.steps = 0;
   return pl;
+}
+
+SmallPlan cart2d_small_step_plan(const int win[4], bool fp64) {
+  const int nx = win[1] - win[0], ny = win[3] - win[2];
+  const SmallPlan pl = plan(nx, ny, fp64, 1);
+  // FP32 tiles whose region takes the threads more than one pass: two smaller ones an SM are faster (shared
+  // memory has room for both; 250^2 4.4 us against 5.2, 169^2, one pass, 4.0 against 3.7)
+  return !fp64 && (pl.tw + 4) * (pl.th + 4) > NT<float> ? plan(nx, ny, fp64, 1, 2) : pl;
 }
 
 cudaError_t launch_cart2d_small(const CartGeom &g, const CartStepArgs &a, const SmallPlan &pl,

@@ -166,6 +166,8 @@ struct SmallPlan {
 };
 // (whether a grid is small does not depend on `most`: the largest tile passes the rule with one step)
 SmallPlan cart2d_small_plan(const CartGeom &g, bool fp64, int most);
+// The tile for one step of a small grid over a window or the whole (the bits do not depend on it).
+SmallPlan cart2d_small_step_plan(const int win[4], bool fp64);
 cudaError_t launch_cart2d_small(const CartGeom &g, const CartStepArgs &a, const SmallPlan &pl,
                                 const double *amp, bool fp64, cudaStream_t st);
 // One step of a small 3-D grid (gks_cart3d_small.cu): the tile (-1: march), for a step that
