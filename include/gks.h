@@ -235,7 +235,8 @@ gks_status gks_adjoint_seed(gks_ctx *ctx, const void *state, void *adj);
  * grad_eps[k] += dV^{n+1}/d eps_{design[k]} . adj_in, with V^{n+1} = L(eps) V^n + s^n.
  * state_n = V^n, state_np1 = V^{n+1} (device, internal layout; needed on the design cells and
  * the probe), adj_in = lambda^{n+1}, adj_out = lambda^n (distinct device buffers),
- * grad_eps: device [nd] doubles.  2-D TM, mu = 1.  adj_in and adj_out start on multiples of two values
+ * grad_eps: device [nd] doubles.  Once a kernel's bounded wait has run out, or a state was not finite
+ * (what the next syncing call reports), what is added is NaN.  2-D TM, mu = 1.  adj_in and adj_out start on multiples of two values
  * (16 bytes suit every kernel).  Asynchronous. */
 gks_status gks_adjoint_step(gks_ctx *ctx, const void *state_n, const void *state_np1,
                             const void *adj_in, void *adj_out, double *grad_eps,

@@ -155,9 +155,8 @@ class DesignProblem:
         self._check()
         return grad
 
-    # The recomputed steps and the lambda march have bounded waits, and one that ran out has to be an error
-    # of this gradient, not of the next forward().  The check waits for the stream, so it comes last (400^2, 350
-    # steps, 8.7 ms a pass: 0.13 ms; before the operations on the gradient were enqueued 0.24).
+    # The recomputed steps and the lambda march have bounded waits.  One that ran out makes the gradient NaN on
+    # the device; it is an error of this gradient, not of the next forward(), wherever the host waits for it.
     def _check(self):
         gks_sync(self.ctx)
 
@@ -165,6 +164,8 @@ class DesignProblem:
         if self.checkpoints is None:
             raise RuntimeError("forward() with keep_checkpoints=True must come first")
         caller = self.torch.cuda.current_stream()
+        if caller == self.stream:
+            return self._backward()
         with self.torch.cuda.stream(self.stream):
             grad = self._backward()
         caller.wait_stream(self.stream)
@@ -228,7 +229,8 @@ def _autograd_class():
         @staticmethod
         def backward(ctx, gJ):
             g = (gJ * ctx.problem._gradient()).to(ctx.dev, ctx.dt)
-            ctx.problem._check()
+            if g.device.type == "cpu":                # the copy has waited; on the device nothing waits
+                ctx.problem._check()
             return g, None
 
     return GKSEnergyObjective

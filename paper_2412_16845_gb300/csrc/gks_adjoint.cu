@@ -130,6 +130,7 @@ struct AdjArgs {
   int perx, pery;
   FaceK<T> fx, fy;
   int wx0, wx1, wy0, wy1;         // lambda^n cells to compute (half open)
+  const int *flag;
 };
 
 __device__ __forceinline__ int wc(int i, int n, int periodic) {
@@ -457,6 +458,7 @@ __global__ void __launch_bounds__(GX * GY) adjoint_post_kernel(const AdjArgs<T> 
   const int slot = in_box ? p.dslot[o] : -1;
   const T en1 = slot >= 0 ? p.Vn1[o] : T(0);
   const double g_old = slot >= 0 ? p.grad[slot] : 0.0;
+  const int failed = __ldcg(p.flag);                    // a wait ran out, or a state was not finite
 #pragma unroll
   for (int i = tid; i < GSX * GSY; i += GX * GY) {
     const int sy = i / GSX, sx = i - sy * GSX;
@@ -500,7 +502,7 @@ __global__ void __launch_bounds__(GX * GY) adjoint_post_kernel(const AdjArgs<T> 
     if (kind != 2) { mu[0] -= fdv(s.lam[0][rsy][rsx], R.eps); mu[1] -= s.lam[hn][rsy][rsx]; mu[2] -= s.lam[ht][rsy][rsx]; }
     gs -= mu[0] * dd[0] + mu[1] * dd[1] + mu[2] * dd[2];
   }
-  p.grad[slot] = g_old + double(gs);
+  p.grad[slot] = failed ? nan("") : g_old + double(gs);  // not a plausible wrong one
 }
 
 // dq/dV for q(V) = dt sum_P |Omega| Ez^2: lam_E[probe] (+)= 2 dt |Omega| Ez.
@@ -578,6 +580,7 @@ cudaError_t adjoint_t(const CartGeom &g, const AdjointArgs &a, cudaStream_t st) 
   p.pw = a.probe_w;
   p.px0 = a.pbox[0]; p.px1 = a.pbox[1]; p.py0 = a.pbox[2]; p.py1 = a.pbox[3];
   p.dt2 = 2.0 * a.dt;
+  p.flag = a.flag;
   p.dx0 = a.dbox[0]; p.dx1 = a.dbox[1]; p.dy0 = a.dbox[2]; p.dy1 = a.dbox[3];
   p.nx = g.nx; p.ny = g.ny;
   p.pitch = g.pitch; p.cstride = g.cstride;
