@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(BX *kBY<T>, 1)
   bool mx, my, rmx, rmy;
   auto column = [&](int cx, int cy, bool &ax, bool &ay) {
     return (int64_t)image8(cy, p.n[1], p.per[1], p.pec[2], p.pec[3], ay) * p.pitch +
-           image8(cx, p.n[0], p.per[0] || cx > p.n[0] + 1, p.pec[0], p.pec[1], ax);
+           image8(cx, p.n[0], p.per[0] | ((unsigned)(cx - p.n[0] - 2) < 64u), p.pec[0], p.pec[1], ax);
   };
   const int64_t own = column(x, y, mx, my);
   const bool ringer = tid < NRING;
