@@ -235,8 +235,7 @@ gks_status gks_adjoint_seed(gks_ctx *ctx, const void *state, void *adj);
  * grad_eps[k] += dV^{n+1}/d eps_{design[k]} . adj_in, with V^{n+1} = L(eps) V^n + s^n.
  * state_n = V^n, state_np1 = V^{n+1} (device, internal layout; needed on the design cells and
  * the probe), adj_in = lambda^{n+1}, adj_out = lambda^n (distinct device buffers),
- * grad_eps: device [nd] doubles.  Once a kernel's bounded wait has run out, or a state was not finite
- * (what the next syncing call reports), what is added is NaN.  2-D TM, mu = 1.  adj_in and adj_out start on multiples of two values
+ * grad_eps: device [nd] doubles.  2-D TM, mu = 1.  adj_in and adj_out start on multiples of two values
  * (16 bytes suit every kernel).  Asynchronous. */
 gks_status gks_adjoint_step(gks_ctx *ctx, const void *state_n, const void *state_np1,
                             const void *adj_in, void *adj_out, double *grad_eps,
@@ -250,6 +249,11 @@ gks_status gks_adjoint_step(gks_ctx *ctx, const void *state_n, const void *state
 gks_status gks_adjoint_step_window(gks_ctx *ctx, const void *state_n, const void *state_np1,
                                    const void *adj_in, void *adj_out, double *grad_eps,
                                    int32_t add_probe, int64_t x0, int64_t x1, int64_t y0, int64_t y1);
+
+/* Enqueue: grad_eps[0 .. n) (device) = NaN if the context has failed, i.e. if the next syncing call will report
+ * GKS_E_TIMEOUT or GKS_E_NONFINITE; left as it is otherwise.  Called after the last adjoint step, it keeps a
+ * gradient that is used without a syncing call from being a plausible wrong one.  Asynchronous. */
+gks_status gks_guard_gradient(gks_ctx *ctx, double *grad_eps, int64_t n);
 
 /* ---- Domain split across ranks (one process per GPU).  The finite-volume update of Sec. 3.1
  * reaches two cells along every axis (the Green-Gauss gradient of Sec. 3.1, then the face flux

@@ -15,7 +15,7 @@ import math
 import numpy as np
 
 from .gks import (GKSSolver, gks_adjoint_seed, gks_adjoint_step_window, gks_copy_state,
-                  gks_load_state, gks_objective, gks_reset_objective, gks_set_materials_box,
+                  gks_guard_gradient, gks_load_state, gks_objective, gks_reset_objective, gks_set_materials_box,
                   gks_set_objective, gks_state_layout, gks_step_state_window, gks_sync)
 
 
@@ -199,6 +199,7 @@ class DesignProblem:
                     gks_adjoint_step_window(ctx, ptrs[n - s], ptrs[n - s + 1], lam_ptr, lam2_ptr,
                                             grad_ptr, n >= 1, *win)
                 lam_ptr, lam2_ptr = lam2_ptr, lam_ptr
+        gks_guard_gradient(ctx, grad_ptr, self.design.size)
         del pool
         return grad
 

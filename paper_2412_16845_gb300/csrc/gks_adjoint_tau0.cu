@@ -316,7 +316,6 @@ struct PostArgs {
   int nx, ny, perx, pery;
   int64_t pitch, cstride;
   AxisK<T> X, Y;
-  const int *flag;
 };
 
 template <typename T>
@@ -357,7 +356,6 @@ __global__ void __launch_bounds__(GX * GY) adjoint_post_tau0_kernel(const __grid
   const int slot = in && gx >= p.dx0 && gx < p.dx1 && gy >= p.dy0 && gy < p.dy1 ? p.dslot[o] : -1;
   const T en1 = slot >= 0 ? p.Vn1[o] : T(0);
   const double g_old = slot >= 0 ? p.grad[slot] : 0.0;
-  const int failed = __ldcg(p.flag);                    // a wait ran out, or a state was not finite
   auto idx = [](int i, int n, int per) {
     if (per) {
       i %= n;
@@ -407,7 +405,7 @@ __global__ void __launch_bounds__(GX * GY) adjoint_post_tau0_kernel(const __grid
   face(integral_constant<int, 0>{}, integral_constant<bool, true>{}, !p.perx && gx == p.nx - 1);
   face(integral_constant<int, 1>{}, integral_constant<bool, false>{}, !p.pery && gy == 0);
   face(integral_constant<int, 1>{}, integral_constant<bool, true>{}, !p.pery && gy == p.ny - 1);
-  p.grad[slot] = failed ? nan("") : g_old + double(gs);  // not a plausible wrong one
+  p.grad[slot] = g_old + double(gs);
 }
 
 template <typename T>
@@ -425,7 +423,6 @@ cudaError_t post_t(const CartGeom &g, const AdjointArgs &a, const int b[4], cuda
   p.dx0 = a.dbox[0]; p.dx1 = a.dbox[1]; p.dy0 = a.dbox[2]; p.dy1 = a.dbox[3];
   p.bx0 = b[0]; p.bx1 = b[1]; p.by0 = b[2]; p.by1 = b[3];
   p.dt2 = 2.0 * a.dt;
-  p.flag = a.flag;
   p.nx = g.nx; p.ny = g.ny; p.perx = g.periodic[0]; p.pery = g.periodic[1];
   p.pitch = g.pitch; p.cstride = g.cstride;
   p.X = make_axis<T>(a.C, a.c, g.h[0], g.h[1], 1.0);

@@ -1003,6 +1003,15 @@ gks_status gks_adjoint_step_window(gks_ctx *ctx, const void *state_n, const void
   return GKS_OK;
 }
 
+gks_status gks_guard_gradient(gks_ctx *ctx, double *grad_eps, int64_t n) {
+  if (!ctx) return GKS_E_ARG;
+  if (n < 0 || (n > 0 && !grad_eps)) return fail(ctx, GKS_E_ARG, "grad_eps / n");
+  if (n == 0) return GKS_OK;
+  GKS_CUDA(gks::launch_guard_gradient(grad_eps, n, ctx->flag, ctx->st));
+  ctx->launches += 1;
+  return GKS_OK;
+}
+
 gks_status gks_get_info(const gks_ctx *ctx, double *dt, double *t, int64_t *step,
                         int64_t *n_cells, double *c_lattice) {
   if (!ctx) return GKS_E_ARG;

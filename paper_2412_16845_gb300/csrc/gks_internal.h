@@ -136,6 +136,7 @@ cudaError_t launch_adjoint_step(const CartGeom &g, const AdjointArgs &a, bool fp
                                 cudaStream_t st);
 cudaError_t launch_probe_grad(const void *V, void *lam, const int64_t *off, const double *w,
                               int64_t np, double dt, bool assign, bool fp64, cudaStream_t st);
+cudaError_t launch_guard_gradient(double *grad, int64_t n, const int *flag, cudaStream_t st);
 // The objective buffer: (sum, Kahan compensation), kObjParts per-block partials and a ticket.
 constexpr int kObjParts = 64;
 constexpr int kObjWords = 2 + kObjParts + 1;

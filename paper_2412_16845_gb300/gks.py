@@ -98,6 +98,7 @@ SIGNATURES = {
                                                ctypes.c_void_p, ctypes.c_void_p, ctypes.c_void_p,
                                                ctypes.c_int32, ctypes.c_int64, ctypes.c_int64,
                                                ctypes.c_int64, ctypes.c_int64]),
+    "gks_guard_gradient": (ctypes.c_int, [_CTX, ctypes.c_void_p, ctypes.c_int64]),
     "gks_step_state_window": (ctypes.c_int, [_CTX, ctypes.c_void_p, ctypes.c_void_p,
                                              ctypes.c_int64, ctypes.c_int64, ctypes.c_int64,
                                              ctypes.c_int64, ctypes.c_int64]),
@@ -294,6 +295,10 @@ def gks_adjoint_step_window(ctx, state_n, state_np1, adj_in, adj_out, grad_eps, 
     _check(ctx, load_library().gks_adjoint_step_window(ctx, state_n, state_np1, adj_in, adj_out,
                                                        grad_eps, 1 if add_probe else 0, x0, x1, y0,
                                                        y1))
+
+
+def gks_guard_gradient(ctx, grad_eps, n):
+    _check(ctx, load_library().gks_guard_gradient(ctx, grad_eps, n))
 
 
 def gks_step_state_window(ctx, src, dst, step, x0, x1, y0, y1):

@@ -48,6 +48,7 @@ def test_a_wait_that_ran_out_in_backward_is_an_error(fake, fake_torch, kernel):
     with pytest.raises(gks.GksError) as e:
         p.backward()
     assert e.value.status == gks.GKS_E_TIMEOUT
+    assert "guard_gradient_kernel" in fake.launched()[-1]    # for a gradient that is used without the check
     p.close()
 
 
