@@ -255,8 +255,8 @@ cudaError_t launch_t(const CartGeom &g, const CartStepArgs &a, cudaStream_t st) 
 // steps of 24 grids of 8^3 to 120^3 cells with every tile, open sides, with and without the limiter.  A tile
 // costs its sides' work; a second FP32 tile on an SM hides the first one's latency unless shared memory holds
 // only one (8 x 8 x 8).  us a step with one, two, four and eight tiles on the busiest SM: FP32 8 x 4 x 4 4.4,
-// 6.9, 8.9, 14.9; 8 x 8 x 8 7.6, 13.9, 26.0, 49.8; FP64 8 x 8 x 4 24.5, 46.3, 93.4, 181; estimates within 10%
-// (FP32 8%, 8 x 4 x 4 alone -4%).  Otherwise: FP32 with open or periodic sides the march (8.1 at 32^3, 10.2 at
+// 6.9, 8.9, 14.9; 8 x 8 x 8 7.6, 13.9, 26.0, 49.8; FP64 8 x 8 x 4 24.5, 46.3, 93.4, 181.  The estimates of the
+// tiles taken are within 11%.  Otherwise: FP32 with open or periodic sides the march (8.1 at 32^3, 10.2 at
 // 48^3: crossing near 100,000 cells); with the limiter or walls the general kernel (18.8 and 22.9; limited small
 // tiles 5.8 and 11.7; crossing near 500,000); FP64 the march (48^3 107, small tiles 70; 130 x 118 x 97 929,
 // small tiles 985).
